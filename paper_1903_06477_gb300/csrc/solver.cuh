@@ -199,8 +199,8 @@ template <typename T>
 struct DevWork {
     IrBufs ir;
     Resume* res;  // loop state handed from the FP32 to the FP64 phase (SCS_MIXED)
-    T* chol;      // direct solves: n x n row-major, lower triangle = Cholesky factor of I + A^T A (else null)
-    int* chol_fail;  // set by MODE_FACTOR if a pivot was not positive (the factor is then not used)
+    T* dinv;      // direct solves: (I + A^T A)^{-1}, n x n (else null)
+    int* dinv_fail;  // set by MODE_FACTOR if a pivot was not positive (the inverse is then not used)
     HV<T> u, ut, ub, Ru, d, dt, wb, Rw, zp, xip, zt;
     T* g;       // n+m: g = M^{-1}(c, b)
     T* ws[2];   // CG warm starts (n) for the u~ and d~ systems
@@ -1037,19 +1037,138 @@ __device__ int cg_loop(Team& tm, const Sell<T>& A, const Sell<T>& AT, int n, CgB
 // ---------------------------------------------------------------------------
 // Direct solves of (I + A^T A) x = b (the "direct" alternative Sec. 4.1 names
 // beside CG), for one CTA per instance: the matrix is formed column by column
-// as e_j + A^T (A e_j) with the solver's own sparse products, factored
-// L L^T in place (right-looking, one column per step), and each solve is a
-// forward and a backward substitution in blocks of 32: warp 0 solves the
-// 32 x 32 diagonal block with shuffles, then the whole CTA updates the rows
-// outside it (two CTA barriers per block).
+// as e_j + A^T (A e_j) with the solver's own sparse products and inverted in
+// place once, at setup; a solve is then one symmetric product.
+//
+// Why the inverse and not its factor L L^T: both take n^2 multiply-adds and
+// n^2 words a solve, but the two triangular solves are a chain of n divisions
+// and 4 n / 32 CTA barriers, and on this GPU an FP64 instruction occupies the
+// SM's FP64 pipe for 16 cycles whether one lane needs it or all 32 do.  The
+// forward error has the same bound, a multiple of n u cond(I + A^T A), and the
+// product is applied to the residual of the warm start (minv).
 // ---------------------------------------------------------------------------
-constexpr int CHOL_B = 32;
+constexpr int DIR_B = 32;  // tile of the inversion: DIR_B^2 values fit each of the two shared arrays
+
+// Blocked symmetric sweep (Gauss-Jordan without pivoting, as SPD allows) of
+// the lower triangle of the n x n row-major matrix L.  Sweeping the block
+// column k, with D = A_kk, P = D^{-1}, C_i = A_ik and W_i = C_i P:
+//   A_ij -= W_i C_j^T (i, j != k),   A_ik = W_i,   A_kk = -P,
+// and after all blocks L = -(input)^{-1}.  n^3 / 2 multiply-adds in 32 x 32
+// tiles; S1 and S2 are DIR_B^2 values of shared memory each.  Returns false if
+// a pivot was not positive (the same Schur complements as a Cholesky factor's).
+template <typename T, class Team>
+__device__ bool direct_sweep(Team& tm, T* L, int n, T* S1, T* S2)
+{
+    const int tid = tm.rank(), nt = tm.size();
+    const int nb = (n + DIR_B - 1) / DIR_B;
+    bool good = true;
+    // tile C_i of block column k, element (r, q), from the lower triangle
+    auto colv = [&](int i, int k, int r, int q) -> T {
+        const int gi = i * DIR_B + r, gk = k * DIR_B + q;
+        if (gi >= n || gk >= n) return T(0);
+        return i > k ? L[(size_t)gi * n + gk] : L[(size_t)gk * n + gi];
+    };
+    for (int k = 0; k < nb; ++k) {
+        const int w = min(DIR_B, n - k * DIR_B);
+        const size_t dk = (size_t)k * DIR_B * (n + 1);  // element (0, 0) of A_kk
+        // P: scalar sweeps of D, alternating between the two arrays (one barrier a pivot)
+        T *cur = S1, *nxt = S2;
+        for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+            const int r = e / DIR_B, c = e % DIR_B;
+            cur[e] = r < w && c < w ? L[dk + (size_t)max(r, c) * n + min(r, c)] : T(r == c ? 1 : 0);
+        }
+        tm.sync();
+        for (int p = 0; p < w; ++p) {
+            const T d = cur[p * DIR_B + p];
+            if (!(d > T(0))) good = false;
+            const T rd = T(1) / (d > T(0) ? d : T(1));
+            for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+                const int r = e / DIR_B, c = e % DIR_B;
+                const T v = cur[e];
+                nxt[e] = r == p ? (c == p ? -rd : v * rd)
+                                : (c == p ? v * rd : v - cur[r * DIR_B + p] * rd * cur[p * DIR_B + c]);
+            }
+            tm.sync();
+            T* t = cur;
+            cur = nxt;
+            nxt = t;
+        }
+        for (int e = tid; e < DIR_B * DIR_B; e += nt) {  // A_kk = -P, whole block
+            const int r = e / DIR_B, c = e % DIR_B;
+            if (r < w && c < w) L[dk + (size_t)r * n + c] = cur[e];
+        }
+        tm.sync();
+        // W_i = C_i P into S1 (C_i staged in S2); P is read back from A_kk
+        auto make_w = [&](int i) {
+            for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+                const int a = e / DIR_B, b = e % DIR_B;  // b along the stored rows
+                const int r = i > k ? a : b, q = i > k ? b : a;
+                S2[r * DIR_B + q] = colv(i, k, r, q);
+            }
+            tm.sync();
+            for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+                const int r = e / DIR_B, c = e % DIR_B;
+                T a0 = 0, a1 = 0;
+                if (c < w)
+                    for (int q = 0; q + 1 < w; q += 2) {
+                        a0 -= S2[r * DIR_B + q] * L[dk + (size_t)q * n + c];
+                        a1 -= S2[r * DIR_B + q + 1] * L[dk + (size_t)(q + 1) * n + c];
+                    }
+                if (c < w && (w & 1)) a0 -= S2[r * DIR_B + w - 1] * L[dk + (size_t)(w - 1) * n + c];
+                S1[e] = a0 + a1;
+            }
+            tm.sync();
+        };
+        for (int i = 0; i < nb; ++i) {
+            if (i == k) continue;
+            make_w(i);
+            for (int j = 0; j <= i; ++j) {
+                if (j == k) continue;
+                // C_j transposed, element (q, c) at q DIR_B + (c xor q): rows and columns both hit distinct banks
+                for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+                    const int a = e / DIR_B, b = e % DIR_B;
+                    const int c = j > k ? a : b, q = j > k ? b : a;
+                    S2[q * DIR_B + (c ^ q)] = colv(j, k, c, q);
+                }
+                tm.sync();
+                for (int e = tid; e < DIR_B * DIR_B / 4; e += nt) {  // four rows r, r + 8, ... of one column a thread
+                    const int r = e / DIR_B, c = e % DIR_B;
+                    T acc[4] = {0, 0, 0, 0};
+                    for (int q = 0; q < w; ++q) {
+                        const T v = S2[q * DIR_B + (c ^ q)];
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) acc[h] = fmaT(S1[(r + 8 * h) * DIR_B + q], v, acc[h]);
+                    }
+                    const int gj = j * DIR_B + c;
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int gi = i * DIR_B + r + 8 * h;
+                        if (gi < n && gj <= gi) L[(size_t)gi * n + gj] -= acc[h];
+                    }
+                }
+                tm.sync();
+            }
+        }
+        for (int i = 0; i < nb; ++i) {  // the block column itself, once nobody needs C any more
+            if (i == k) continue;
+            make_w(i);
+            for (int e = tid; e < DIR_B * DIR_B; e += nt) {
+                const int a = e / DIR_B, b = e % DIR_B;
+                const int r = i > k ? a : b, q = i > k ? b : a;
+                const int gi = i * DIR_B + r, gk = k * DIR_B + q;
+                if (gi < n && gk < n) L[i > k ? (size_t)gi * n + gk : (size_t)gk * n + gi] = S1[r * DIR_B + q];
+            }
+            tm.sync();
+        }
+    }
+    return good;
+}
 
 template <typename T, class Team>
-__device__ void chol_factor(Team& tm, const DevProb<T>& P, const DevWork<T>& W)
+__device__ void direct_setup(Team& tm, const DevProb<T>& P, const DevWork<T>& W, double* s1, double* s2)
 {
     const int n = P.n;
-    T* L = W.chol;
+    T* L = W.dinv;
     T* ej = W.cp;
     T* y = W.tm;
     for (int j = 0; j < n; ++j) {
@@ -1062,97 +1181,64 @@ __device__ void chol_factor(Team& tm, const DevProb<T>& P, const DevWork<T>& W)
         });
         tm.sync();
     }
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int j = 0; j < n; ++j) {
-        if (threadIdx.x == 0) {
-            const T djj = L[(size_t)j * n + j];
-            if (!(djj > T(0))) bad = 1;
-            L[(size_t)j * n + j] = djj > T(0) ? sqrt(djj) : T(1);
+    const bool good = direct_sweep<T>(tm, L, n, reinterpret_cast<T*>(s1), reinterpret_cast<T*>(s2));
+    // both triangles, so that a solve reads rows: the sweep left minus the inverse in the lower one
+    for (int i = tm.rank() >> 5; i < n; i += tm.size() >> 5)
+        for (int j = threadIdx.x & 31; j <= i; j += 32) {
+            const T v = -L[(size_t)i * n + j];
+            L[(size_t)i * n + j] = v;
+            L[(size_t)j * n + i] = v;
         }
-        __syncthreads();
-        const T d = L[(size_t)j * n + j];
-        for (int i = j + 1 + tm.rank(); i < n; i += tm.size()) L[(size_t)i * n + j] /= d;
-        __syncthreads();
-        const int r = n - j - 1;
-        for (long long idx = tm.rank(); idx < (long long)r * r; idx += tm.size()) {
-            const int ii = j + 1 + (int)(idx / r), kk = j + 1 + (int)(idx % r);
-            if (kk <= ii) L[(size_t)ii * n + kk] -= L[(size_t)ii * n + j] * L[(size_t)kk * n + j];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && bad) atomicExch(W.chol_fail, 1);
-    __syncthreads();
+    if (threadIdx.x == 0 && !good) atomicExch(W.dinv_fail, 1);
+    tm.sync();
 }
 
-// b (n, in place) <- (L L^T)^{-1} b.  dg: CHOL_B x CHOL_B values of shared
-// memory for the diagonal block, loaded by the whole CTA with coalesced reads
-// before warp 0 solves it; element (r, c) sits at r CHOL_B + (c xor r), so the
-// lanes of a warp reading one column, or one row, hit distinct banks.  zb:
-// CHOL_B values of shared memory.
+// x += D r with the symmetric inverse D: column j belongs to one thread, whose
+// warp reads 32 consecutive words of each row; the rows are cut into as many
+// parts as there are idle warps (n below the CTA's size), added through shared
+// memory (part: up to DIR_PART values).  Bound by the FP64 pipe (n^2 / 2
+// cycles an SM) or by reading D from L2.  1024 portfolio instances of 20 to
+// 400 columns, 20 iterations in FP64: 24.3 ms with the triangular solves.
+constexpr int DIR_PART = 1024;
+
 template <typename T, class Team>
-__device__ void chol_solve(Team& tm, const T* L, int n, T* b, T* dg, T* zb)
+__device__ void direct_solve(Team& tm, const T* D, int n, const T* r, T* x, T* part)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    auto D = [&](int r, int c) -> T& { return dg[r * CHOL_B + (c ^ r)]; };
-    auto load_diag = [&](int jb, int w) {
-        __syncthreads();  // the previous block's readers are done
-        for (int idx = threadIdx.x; idx < w * CHOL_B; idx += blockDim.x) {
-            const int r = idx / CHOL_B, c = idx % CHOL_B;
-            D(r, c) = c < w ? L[(size_t)(jb + r) * n + jb + c] : T(0);
+    const int np = (n + 31) & ~31;  // columns, whole warps
+    const int parts = max(1, min(tm.size() / np, DIR_PART / np));
+    if (parts == 1) {
+        for (int j = tm.rank(); j < n; j += tm.size()) {
+            T a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            const T* d = D + j;
+            int i = 0;
+            for (; i + 8 <= n; i += 8)
+#pragma unroll
+                for (int h = 0; h < 8; ++h) a[h] = fmaT(d[(size_t)(i + h) * n], r[i + h], a[h]);
+            for (; i < n; ++i) a[0] = fmaT(d[(size_t)i * n], r[i], a[0]);
+            x[j] += ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
         }
-        __syncthreads();
-    };
-    // forward: L z = b
-    for (int jb = 0; jb < n; jb += CHOL_B) {
-        const int w = min(CHOL_B, n - jb);
-        load_diag(jb, w);
-        if (warp == 0) {
-            T v = lane < w ? b[jb + lane] : T(0);
-            for (int c = 0; c < w; ++c) {
-                const T zc = __shfl_sync(FULL_MASK, v, c) / D(c, c);
-                if (lane == c) v = zc;
-                if (lane > c && lane < w) v -= D(lane, c) * zc;
-            }
-            if (lane < w) {
-                b[jb + lane] = v;
-                zb[lane] = v;
-            }
-        }
-        __syncthreads();
-        for (int i = jb + w + tm.rank(); i < n; i += tm.size()) {
-            T acc = b[i];
-            const T* row = L + (size_t)i * n + jb;
-            for (int c = 0; c < w; ++c) acc -= row[c] * zb[c];
-            b[i] = acc;
-        }
-        __syncthreads();
+        tm.sync();
+        return;
     }
-    // backward: L^T x = z
-    for (int jb = ((n - 1) / CHOL_B) * CHOL_B; jb >= 0; jb -= CHOL_B) {
-        const int w = min(CHOL_B, n - jb);
-        load_diag(jb, w);
-        if (warp == 0) {
-            T v = lane < w ? b[jb + lane] : T(0);
-            for (int c = w - 1; c >= 0; --c) {
-                const T xc = __shfl_sync(FULL_MASK, v, c) / D(c, c);
-                if (lane == c) v = xc;
-                if (lane < c) v -= D(c, lane) * xc;
-            }
-            if (lane < w) {
-                b[jb + lane] = v;
-                zb[lane] = v;
-            }
-        }
-        __syncthreads();
-        for (int k = tm.rank(); k < jb; k += tm.size()) {
-            T acc = b[k];
-            for (int c = 0; c < w; ++c) acc -= L[(size_t)(jb + c) * n + k] * zb[c];
-            b[k] = acc;
-        }
-        __syncthreads();
+    const int g = tm.rank() / np, j = tm.rank() % np;
+    if (g < parts && j < n) {
+        const int i1 = (int)((long long)n * (g + 1) / parts);
+        int i = (int)((long long)n * g / parts);
+        T a[4] = {0, 0, 0, 0};
+        const T* d = D + j;
+        for (; i + 4 <= i1; i += 4)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) a[h] = fmaT(d[(size_t)(i + h) * n], r[i + h], a[h]);
+        for (; i < i1; ++i) a[0] = fmaT(d[(size_t)i * n], r[i], a[0]);
+        part[g * np + j] = (a[0] + a[1]) + (a[2] + a[3]);
     }
+    tm.sync();
+    for (int k = tm.rank(); k < n; k += tm.size()) {
+        T s = part[k];
+        for (int h = 1; h < parts; ++h) s += part[h * np + k];
+        x[k] += s;
+    }
+    tm.sync();
 }
 
 // ---------------------------------------------------------------------------
@@ -1165,7 +1251,7 @@ template <typename T, class Team>
 __device__ __forceinline__ bool direct_available(const Team&, const DevWork<T>& W)
 {
     if constexpr (Team::kGrid) return false;
-    else return W.chol != nullptr;
+    else return W.dinv != nullptr;
 }
 
 template <typename T, class Team>
@@ -1195,14 +1281,9 @@ __device__ int minv(Team& tm, const DevProb<T>& P, const DevWork<T>& W, const T*
         for (int j = tm.rank(); j < n; j += tm.size()) x[j] = 0;
         tm.sync();
     } else if (direct_available(tm, W)) {
-        // direct: x <- x + (L L^T)^{-1} r, the residual of the warm start solved exactly
-        if constexpr (!Team::kGrid) {
-            // shared scratch of the CTA: the AA direction's Cholesky array (idle during a linear
-            // solve) for the diagonal block, the reduction rows for the block's solution
-            chol_solve<T>(tm, W.chol, n, r, reinterpret_cast<T*>(tm.scratch), reinterpret_cast<T*>(tm.red));
-        }
-        for (int j = tm.rank(); j < n; j += tm.size()) x[j] += r[j];
-        tm.sync();
+        // direct: the residual of the warm start solved exactly; the shared scratch is the AA
+        // direction's Cholesky array, idle during a linear solve
+        if constexpr (!Team::kGrid) direct_solve<T>(tm, W.dinv, n, r, x, reinterpret_cast<T*>(tm.scratch));
     } else if (sqrt(rr) > tol) {
         const unsigned long long tc0 = tm.leader() ? gtimer() : 0ull;
         it = cg_loop<T>(tm, P.A, P.AT, n, CgBufs<T>{r, W.cp, W.cq, tmv}, x, rr, tol, cg_max);
@@ -3019,7 +3100,7 @@ __device__ void run_mode(Team& tm, const DevProb<T>& P, const DevWork<T>& W, con
     const int n = P.n, m = P.m, nm = n + m;
     if (mode == MODE_FACTOR) {
         if constexpr (!Team::kGrid) {
-            if (W.chol) chol_factor(tm, P, W);
+            if (W.dinv) direct_setup(tm, P, W, G, sm_L);
         }
         return;
     }
