@@ -44,13 +44,19 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) k_grid(const __grid_constant_
     run_mode<T>(tm, a.P, a.W, a.S, a.mode, a.slot, sf.G, sf.rhs, sf.L, sf.t, dyn);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(1024) k_block(const Args<T>* insts, int B, int* queue, DevSettings S, int mode)
+// One CTA per instance, persistent over a queue.  MAXT is the largest block:
+// up to BLOCK_SMALL threads the kernel is built for BLOCK_SMALL_CTAS resident
+// CTAs of that size, which leaves a thread 128 registers; built for 1024
+// threads it has 64 and the solver's functions spill 9 KB of stores a thread
+// (ptxas -v, FP64).  Which one runs is block_kernel's choice.
+template <typename T, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == BLOCK_SMALL ? BLOCK_SMALL_CTAS : 1)
+    k_block(const Args<T>* insts, int B, int* queue, DevSettings S, int mode)
 {
     __shared__ SmemFixed sf;
     __shared__ int sidx;
     extern __shared__ __align__(128) unsigned char dyn[];
-    BlockTeam tm{sf.red, nullptr, sf.mbar, sf.ph, nullptr, sf.L};
+    BlockTeam<MAXT> tm{sf.red, nullptr, sf.mbar, sf.ph, nullptr, sf.L};
     for (;;) {
         if (threadIdx.x == 0) sidx = atomicAdd(queue, 1);
         __syncthreads();
@@ -72,14 +78,7 @@ __global__ void k_convert(const Tin* in, Tout* out, long long n)
 
 template <typename T>
 const void* kgrid_ptr() { return (const void*)k_grid<T>; }
-template <typename T>
-const void* kblock_ptr() { return (const void*)k_block<T>; }
-template <typename T>
-cudaError_t launch_block(int grid, int threads, size_t dyn, cudaStream_t st, const Args<T>* insts, int B, int* queue,
-                         const DevSettings& S, int mode)
-{
-    k_block<T><<<grid, threads, dyn, st>>>(insts, B, queue, S, mode);
-    return cudaGetLastError();
-}
+template <typename T, int MAXT>
+const void* kblock_build() { return (const void*)k_block<T, MAXT>; }
 
 }  // namespace sscs

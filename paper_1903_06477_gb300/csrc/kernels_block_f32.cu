@@ -1,8 +1,6 @@
-// kernels_block_f32.cu -- FP32 instantiation of the block-team kernel.
+// kernels_block_f32.cu -- FP32 instantiation of the block-team kernel for blocks of up to 1024 threads.
 #include "kernels.cuh"
 
 namespace sscs {
-template const void* kblock_ptr<float>();
-template cudaError_t launch_block<float>(int, int, size_t, cudaStream_t, const Args<float>*, int, int*,
-                                         const DevSettings&, int);
+template const void* kblock_build<float, BLOCK_LARGE>();
 }  // namespace sscs

@@ -1,4 +1,5 @@
-// kernels_block_f64.cu -- FP64 instantiation of the block-team (one CTA per instance) kernel.
+// kernels_block_f64.cu -- FP64 instantiation of the block-team (one CTA per instance) kernel
+// for blocks of up to 1024 threads, and the batches' small kernels.
 #include "kernels.cuh"
 
 namespace sscs {
@@ -57,9 +58,7 @@ __global__ void k_batch_pack(const Args<double>* a64, int B, const long long* of
     }
 }
 
-template const void* kblock_ptr<double>();
-template cudaError_t launch_block<double>(int, int, size_t, cudaStream_t, const Args<double>*, int, int*,
-                                          const DevSettings&, int);
+template const void* kblock_build<double, BLOCK_LARGE>();
 
 cudaError_t launch_batch_handoff(const Args<float>* a32, const Args<double>* a64, int B, int mem, int resume,
                                  cudaStream_t st)

@@ -34,9 +34,9 @@ __device__ __forceinline__ void block_partial(double (&v)[K], double* red)
     __syncthreads();
 }
 
-// The same sums with fewer FP64 instructions, used by the grid team (in the
-// batch kernel, limited to 64 registers a thread, the larger code made the
-// compiler outline the solver loop with more spills).
+// The same sums with fewer FP64 instructions, used by the grid team and the
+// block team's 128-register build (limited to 64 registers a thread, the
+// larger code made the compiler outline the solver loop with more spills).
 //
 // Each warp's sum of value k is the butterfly tree of warp_sum (pairs of
 // lanes l, l+16, then l, l+8, ..., l, l+1, as seen from lane 0), but the
@@ -81,6 +81,7 @@ __device__ __forceinline__ void block_partial_packed(double (&v)[K], double* red
     __syncthreads();
 }
 
+template <int MAXT>
 struct BlockTeam {
     static constexpr bool kGrid = false;
     double* red;
@@ -101,7 +102,10 @@ struct BlockTeam {
     template <int K>
     __device__ __forceinline__ void reduce(double (&v)[K])
     {
-        block_partial<K>(v, red);
+        if constexpr (MAXT <= BLOCK_SMALL)
+            block_partial_packed<K>(v, red);
+        else
+            block_partial<K>(v, red);
         const int nw = blockDim.x >> 5;
         if (threadIdx.x < K) {
             double s = 0.0;
