@@ -11,8 +11,8 @@ constexpr int KMAX = 16;                       // max values in one team reducti
 constexpr int MAX_WARPS = 32;                  // 1024 threads per block at most
 constexpr int GRID_THREADS = 512;              // largest block of the grid team (one CTA per SM)
 constexpr int BLOCK_LARGE = 1024;              // largest block of the block team
-constexpr int BLOCK_SMALL = 256;               // largest block of its 128-register build
-constexpr int BLOCK_SMALL_CTAS = 2;            // resident CTAs of that size
+constexpr int BLOCK_SMALL = 512;               // largest block of its 128-register build
+constexpr int BLOCK_SMALL_CTAS = 1;            // resident CTAs of that size
 constexpr int CB_MAX_STAGES = 4;               // deepest copy ring of the column-blocked products
 constexpr unsigned long long BARRIER_TIMEOUT_NS = 10ull * 1000ull * 1000ull * 1000ull;  // 10 s
 

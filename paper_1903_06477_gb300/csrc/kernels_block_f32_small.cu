@@ -1,4 +1,4 @@
-// kernels_block_f32_small.cu -- FP32 instantiation of the block-team kernel for blocks of up to 256 threads.
+// kernels_block_f32_small.cu -- FP32 instantiation of the block-team kernel for blocks of up to 512 threads.
 #include "kernels.cuh"
 
 namespace sscs {

@@ -1,4 +1,4 @@
-// kernels_block_f64_small.cu -- FP64 instantiation of the block-team kernel for blocks of up to 256 threads.
+// kernels_block_f64_small.cu -- FP64 instantiation of the block-team kernel for blocks of up to 512 threads.
 #include "kernels.cuh"
 
 namespace sscs {

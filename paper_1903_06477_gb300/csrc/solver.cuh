@@ -18,7 +18,6 @@ namespace sscs {
 constexpr int MAXMEM = 64;   // direction memory cap (RB)
 constexpr int AAMAX = 32;    // Anderson memory cap (Gram matrix kept in shared memory)
 constexpr int PSD_MAX = 64;  // largest PSD order decomposed in shared memory
-constexpr int PSD_LD = PSD_MAX + 1;  // row stride bound of a block's matrices in shared memory
 constexpr int PSD_BIG_MAX = 1024;    // largest PSD order (orders above PSD_MAX use a global-memory workspace)
 
 enum Mode { MODE_SETUP = 0, MODE_SOLVE = 1, MODE_LINSYS = 2, MODE_PROJECT = 3, MODE_APPLY_T = 4, MODE_PROFILE = 5,
@@ -181,7 +180,7 @@ struct DevProb {
     int ep, ed;        // primal / dual exponential cones (3 rows each)
     int e_off;         // row offset of the first exponential cone inside s
     // PSD blocks above PSD_MAX: the Jacobi workspace of block k starts at psd_big + big_off[k]
-    // bytes (laid out by psd_big_ws below; big_off[k] < 0 for blocks decomposed in shared memory)
+    // bytes (laid out by psd_layout below; big_off[k] < 0 for blocks decomposed in shared memory)
     unsigned char* psd_big;
     const long long* big_off;
     const long long* v_off;  // byte offset of each PSD block's warm-start eigenvectors in DevWork::psd_v
@@ -1198,7 +1197,8 @@ __device__ void direct_setup(Team& tm, const DevProb<T>& P, const DevWork<T>& W,
 // parts as there are idle warps (n below the CTA's size), added through shared
 // memory (part: up to DIR_PART values).  Bound by the FP64 pipe (n^2 / 2
 // cycles an SM) or by reading D from L2.  1024 portfolio instances of 20 to
-// 400 columns, 20 iterations in FP64: 24.3 ms with the triangular solves.
+// 400 columns, 20 iterations in FP64: 24.3 ms with the triangular solves, 17.4
+// ms so; one instance of 560 columns, 16 iterations: 23.9 and 14.4 ms.
 constexpr int DIR_PART = 1024;
 
 template <typename T, class Team>
@@ -1466,97 +1466,245 @@ __device__ __forceinline__ double block_sum(double x, double* red)
     return s;
 }
 
-// Parallel two-sided Jacobi (round-robin pairing, d/2 disjoint rotations per
-// round) on the dp x dp matrix X in shared memory; V receives the
-// eigenvectors as columns.  Rotation formula as in the textbook cyclic method.
-// v_init: V already holds an orthogonal start basis (the rotations are
-// accumulated onto it), else it starts as the identity.  Returns true if the
-// off-diagonal mass fell below tol2 times the total within max_sweeps (the
-// same value in every thread).
+// Parallel two-sided Jacobi (round-robin pairing, dp/2 disjoint rotations per
+// round) on the symmetric dp x dp matrix X (its lower triangle, row stride ld =
+// dp + 1, odd, so that a warp walking a column touches 32 banks); V receives
+// the eigenvectors as columns.  v_init: V already holds an orthogonal start
+// basis (the rotations are accumulated onto it), else it starts as the
+// identity.  Returns true if the off-diagonal mass fell below tol2 times the
+// total within max_sweeps (the same value in every thread); X's diagonal then
+// holds the eigenvalues.
+//
+// One CTA barrier a round: the pairs of a round cut X into 2 x 2 blocks (pair
+// k's rows, pair l's columns), each updated from both sides by one thread, and
+// the block that holds the next round's pair k also computes that pair's
+// rotation once it is updated, into the other of two rotation buffers.  (The
+// pairs of round r+1 are (r+1+k, r+1-k), whose members lie in pairs k+1 and
+// k-1 of round r.)  With separate passes for rotations, columns and rows a
+// round took three barriers and updated both triangles: four projections of 512
+// FP32 blocks of order 64 10.0 ms, now 6.5 ms; six FP64 iterations with 150
+// blocks of order 20 to 63 32.6 ms, now 20.8 ms; four with one block of order
+// 120 129 ms, now 76 ms.
+//
+// FP64: the FP64 pipe (2 multiply-adds a cycle and SM) is the bound, so the
+// rotations are applied in scaled form (fast Givens): X = D X^ D and V = V^ D
+// with D diagonal, x^_p -= al x^_q, x^_q += be x^_p -- one multiply-add per
+// element instead of a product and a multiply-add -- and D is multiplied in
+// after each sweep (its entries shrink by at most sqrt(2) a round).  The angle
+// is found in FP32 -- any t with c = 1/sqrt(1 + t^2), s = t c is a rotation,
+// and c, the scales and the diagonal are FP64 for the t that was taken; an
+// angle 1e-7 off leaves 1e-7 of the element for the next sweep.  Per round
+// dp^2 + dp^2 / 2 multiply-adds against 3 dp^2 products and multiply-adds.
 template <typename T>
-__device__ bool jacobi_block(T* X, T* V, int dp, int ld, int* pp, int* qq, T* cs, T* sn, double* red, double tol2,
-                             int max_sweeps, bool v_init = false)
+struct JacobiScratch {
+    T *r0, *r1;         // rotations of a round, two buffers of dp/2: (c, s), or (al, be) in FP64
+    T *dg, *sc, *isc;   // FP64: the diagonal of X, the scales D and 1 / D (dp each)
+    static constexpr int words(int dp) { return 5 * dp; }
+    __device__ JacobiScratch(T* base, int dp) : r0(base), r1(base + dp), dg(base + 2 * dp), sc(base + 3 * dp), isc(base + 4 * dp) {}
+};
+
+// block idx of a round (half >= 3): the first `half` hold next round's pairs, see jacobi_block
+__device__ __forceinline__ void jacobi_cell(int idx, int half, int& k, int& l)
 {
-    // X and V are dp x dp with row stride ld = dp + 1 (odd): a warp walking a
-    // column touches 32 different banks
-    const int tid = threadIdx.x, nt = blockDim.x;
-    if (!v_init)
-        for (int idx = tid; idx < dp * dp; idx += nt) {
-            const int i = idx / dp, j = idx % dp;
-            V[i * ld + j] = (i == j) ? T(1) : T(0);
-        }
+    if (idx < half) {
+        k = min(idx + 1, half - 1);
+        l = idx == half - 1 ? half - 2 : max(idx - 1, 0);
+        return;
+    }
+    idx -= half;
+    if (idx < half - 3) {  // neighbours (k - l = 1) but the first and the last
+        k = idx + 2;
+        l = idx + 1;
+        return;
+    }
+    idx -= half - 3;  // k - l >= 3: a triangle
+    int r = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+    while ((r + 1) * (r + 2) / 2 <= idx) ++r;
+    while (r * (r + 1) / 2 > idx) --r;
+    k = r + 3;
+    l = idx - r * (r + 1) / 2;
+}
+
+template <typename T>
+__device__ bool jacobi_block(T* X, T* V, int dp, int ld, T* scratch, double* red, double tol2, int max_sweeps,
+                             bool v_init = false)
+{
+    constexpr bool kFast = sizeof(T) == 8;
+    const JacobiScratch<T> S(scratch, dp);
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    const int half = dp / 2, ncell = half * (half - 1) / 2;
     double total = 0.0;
-    for (int idx = tid; idx < dp * dp; idx += nt) {
-        const T x = X[(idx / dp) * ld + idx % dp];
-        total += (double)x * (double)x;
+    for (int i = warp; i < dp; i += nw) {
+        for (int j = lane; j < i; j += 32) total += 2.0 * (double)X[i * ld + j] * (double)X[i * ld + j];
+        if (lane == 0) total += (double)X[i * ld + i] * (double)X[i * ld + i];
+        if (!v_init)
+            for (int j = lane; j < dp; j += 32) V[i * ld + j] = (i == j) ? T(1) : T(0);
     }
-    __syncthreads();
+    if constexpr (kFast)
+        for (int i = tid; i < dp; i += nt) {
+            S.dg[i] = X[i * ld + i];
+            S.sc[i] = S.isc[i] = T(1);
+        }
     total = block_sum(total, red);
-    const int half = dp / 2;
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        double off = 0.0;
-        for (int idx = tid; idx < dp * dp; idx += nt) {
-            const int i = idx / dp, j = idx % dp;
-            if (i != j) off += (double)X[i * ld + j] * (double)X[i * ld + j];
+    // FP64: a power of two that brings the matrix to about 1, for the FP32 angles
+    const double unit = kFast && total > 0.0 && isfinite(total) ? scalbn(1.0, -ilogb(sqrt(total))) : 1.0;
+    auto pair = [&](int k, int rnd, int& p, int& q) {  // pair k of a round, p < q
+        int a = rnd, b = dp - 1;
+        if (k > 0) {
+            a = rnd + k;
+            if (a >= dp - 1) a -= dp - 1;
+            b = rnd - k;
+            if (b < 0) b += dp - 1;
         }
-        off = block_sum(off, red);
-        if (off <= tol2 * total || off == 0.0) return true;
+        p = min(a, b);
+        q = max(a, b);
+    };
+    auto at = [&](int i, int j) { return i > j ? i * ld + j : j * ld + i; };
+    // the rotation of pair k of a round into buffer buf, applied to the pair's own 2 x 2 block
+    auto rotate = [&](int k, int rnd, int buf) {
+        int p, q;
+        pair(k, rnd, p, q);
+        if constexpr (kFast) {
+            const T dp_ = S.sc[p], dq = S.sc[q], ep = S.isc[p], eq = S.isc[q], app = S.dg[p], aqq = S.dg[q];
+            const T apq = X[q * ld + p] * (dp_ * dq), diff = aqq - app;
+            const float den = (float)(apq * unit), num = (float)(diff * unit);
+            float tf = 0.f;
+            if (den != 0.f) {
+                const float th = num / (2.f * den), at_ = fabsf(th);
+                tf = at_ > 1e18f ? 0.5f / th : copysignf(1.f, th) / (at_ + sqrtf(th * th + 1.f));
+            }
+            const T t = (T)tf, a = fma(t, t, T(1));
+            T c = (T)rsqrtf((float)a);  // two Newton steps to 1 / sqrt(1 + t^2)
+            c = c * fma(T(-0.5) * a * c, c, T(1.5));
+            c = c * fma(T(-0.5) * a * c, c, T(1.5));
+            const T ic = a * c, h = c * c;
+            const T del = h * t * (t * diff - T(2) * apq);
+            S.r0[buf * half + k] = t * dq * ep;
+            S.r1[buf * half + k] = t * dp_ * eq;
+            S.dg[p] = app + del;
+            S.dg[q] = aqq - del;
+            S.sc[p] = c * dp_;
+            S.sc[q] = c * dq;
+            S.isc[p] = ic * ep;
+            S.isc[q] = ic * eq;
+            X[q * ld + p] = h * (fma(-t, t, T(1)) * apq - t * diff) * (ic * ep) * (ic * eq);
+        } else {
+            const T app = X[p * ld + p], aqq = X[q * ld + q], apq = X[q * ld + p];
+            T c = 1, s = 0;
+            if (apq != T(0)) {
+                const T theta = (aqq - app) / (T(2) * apq);
+                const T at_ = theta < T(0) ? -theta : theta;
+                T t;
+                if (at_ > T(1e18))
+                    t = T(0.5) / theta;
+                else
+                    t = (theta >= T(0) ? T(1) : T(-1)) / (at_ + sqrt(theta * theta + T(1)));
+                c = T(1) / sqrt(t * t + T(1));
+                s = t * c;
+            }
+            S.r0[buf * half + k] = c;
+            S.r1[buf * half + k] = s;
+            const T xpp = c * app - s * apq, xpq = s * app + c * apq;  // columns, then rows
+            const T xqp = c * apq - s * aqq, xqq = s * apq + c * aqq;
+            X[p * ld + p] = c * xpp - s * xqp;
+            X[q * ld + p] = c * xpq - s * xqq;
+            X[q * ld + q] = s * xpq + c * xqq;
+        }
+    };
+    // (x_p, x_q) through one rotation
+    auto turn = [](T& xp, T& xq, T r0, T r1) {
+        const T a = xp, b = xq;
+        if constexpr (kFast) {
+            xp = fma(-r0, b, a);
+            xq = fma(r1, a, b);
+        } else {
+            xp = r0 * a - r1 * b;
+            xq = r1 * a + r0 * b;
+        }
+    };
+    int kc[2] = {0, 0}, lc[2] = {0, 0};  // this thread's first two cells
+    if (half >= 3) {
+        if (tid < ncell) jacobi_cell(tid, half, kc[0], lc[0]);
+        if (tid + nt < ncell) jacobi_cell(tid + nt, half, kc[1], lc[1]);
+    } else {
+        kc[0] = 1;
+    }
+    const bool wide = nt >= dp;  // V: a thread has one row and every ng-th pair, or all pairs of several rows
+    const int vi0 = wide ? tid % dp : tid, vstep = wide ? dp : nt, ng = wide ? nt / dp : 1, vg = wide ? tid / dp : 0;
+    bool conv = false;
+    for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
+        double off = 0.0;
+        for (int i = warp; i < dp; i += nw) {
+            if constexpr (kFast) {
+                const T di = S.sc[i];
+                for (int j = lane; j < i; j += 32) {
+                    const T x = X[i * ld + j] * (di * S.sc[j]);
+                    X[i * ld + j] = x;
+                    off += x * x;
+                }
+                if (sweep > 0)
+                    for (int j = lane; j < dp; j += 32) V[i * ld + j] *= S.sc[j];
+            } else {
+                for (int j = lane; j < i; j += 32) off += (double)X[i * ld + j] * (double)X[i * ld + j];
+            }
+        }
+        off = 2.0 * block_sum(off, red);
+        conv = off <= tol2 * total || off == 0.0;
+        if (conv || sweep == max_sweeps) break;
+        if constexpr (kFast) {
+            for (int i = tid; i < dp; i += nt) S.sc[i] = S.isc[i] = T(1);
+            __syncthreads();
+        }
+        for (int k = tid; k < half; k += nt) rotate(k, 0, 0);
+        __syncthreads();
         for (int rnd = 0; rnd < dp - 1; ++rnd) {
-            for (int k = tid; k < half; k += nt) {
-                int a, b;
-                if (k == 0) {
-                    a = rnd;
-                    b = dp - 1;
+            const T* r0 = S.r0 + (rnd & 1) * half;
+            const T* r1 = S.r1 + (rnd & 1) * half;
+            for (int idx = tid, n = 0; idx < ncell; idx += nt, ++n) {
+                int k, l, pk, qk, pl, ql;
+                if (n < 2) {
+                    k = n == 0 ? kc[0] : kc[1];
+                    l = n == 0 ? lc[0] : lc[1];
                 } else {
-                    a = (rnd + k) % (dp - 1);
-                    b = (rnd - k + dp - 1) % (dp - 1);
+                    jacobi_cell(idx, half, k, l);
                 }
-                const int p = a < b ? a : b, qd = a < b ? b : a;
-                const T apq = X[p * ld + qd];
-                T c = 1, s = 0;
-                if (apq != T(0)) {
-                    const T theta = (X[qd * ld + qd] - X[p * ld + p]) / (T(2) * apq);
-                    const T at = theta < T(0) ? -theta : theta;
-                    T t;
-                    if (at > T(1e18))
-                        t = T(0.5) / theta;
-                    else
-                        t = (theta >= T(0) ? T(1) : T(-1)) / (at + sqrt(theta * theta + T(1)));
-                    c = T(1) / sqrt(t * t + T(1));
-                    s = t * c;
+                pair(k, rnd, pk, qk);
+                pair(l, rnd, pl, ql);
+                const T ck = r0[k], sk = r1[k], cl = r0[l], sl = r1[l];
+                const int ia = at(pk, pl), ib = at(pk, ql), ic = at(qk, pl), id = at(qk, ql);
+                T xa = X[ia], xb = X[ib], xc = X[ic], xd = X[id];
+                turn(xa, xb, cl, sl);
+                turn(xc, xd, cl, sl);
+                turn(xa, xc, ck, sk);
+                turn(xb, xd, ck, sk);
+                X[ia] = xa;
+                X[ib] = xb;
+                X[ic] = xc;
+                X[id] = xd;
+                if (idx < half && rnd + 1 < dp - 1) {
+                    rotate(idx, rnd + 1, (rnd + 1) & 1);
+                    if (half == 2) rotate(1, rnd + 1, (rnd + 1) & 1);
                 }
-                pp[k] = p;
-                qq[k] = qd;
-                cs[k] = c;
-                sn[k] = s;
             }
-            __syncthreads();
-            // columns: X <- X J and V <- V J
-            for (int idx = tid; idx < half * dp; idx += nt) {
-                const int k = idx / dp, i = idx % dp;
-                const int p = pp[k], qd = qq[k];
-                const T c = cs[k], s = sn[k];
-                const T xp = X[i * ld + p], xq = X[i * ld + qd];
-                X[i * ld + p] = c * xp - s * xq;
-                X[i * ld + qd] = s * xp + c * xq;
-                const T vp = V[i * ld + p], vq = V[i * ld + qd];
-                V[i * ld + p] = c * vp - s * vq;
-                V[i * ld + qd] = s * vp + c * vq;
-            }
-            __syncthreads();
-            // rows: X <- J^T X
-            for (int idx = tid; idx < half * dp; idx += nt) {
-                const int k = idx / dp, j = idx % dp;
-                const int p = pp[k], qd = qq[k];
-                const T c = cs[k], s = sn[k];
-                const T xp = X[p * ld + j], xq = X[qd * ld + j];
-                X[p * ld + j] = c * xp - s * xq;
-                X[qd * ld + j] = s * xp + c * xq;
-            }
+            for (int i = vi0; i < dp; i += vstep)
+                for (int k = vg; k < half && vg < ng; k += ng) {
+                    int p, q;
+                    pair(k, rnd, p, q);
+                    const T c = r0[k], s = r1[k];
+                    if (kFast && c == T(0) && s == T(0)) continue;
+                    T vp = V[i * ld + p], vq = V[i * ld + q];
+                    turn(vp, vq, c, s);
+                    V[i * ld + p] = vp;
+                    V[i * ld + q] = vq;
+                }
             __syncthreads();
         }
     }
-    return false;
+    if constexpr (kFast) {
+        for (int i = tid; i < dp; i += nt) X[i * ld + i] = S.dg[i];
+        __syncthreads();
+    }
+    return conv;
 }
 
 // ---------------------------------------------------------------------------
@@ -1575,7 +1723,8 @@ __device__ bool jacobi_block(T* X, T* V, int dp, int ld, int* pp, int* qq, T* cs
 // to full precision, and the nearest of the candidates (origin, face point,
 // ray points) is returned.  On the 240 cones of an l1-logistic problem (one
 // CTA) a projection took 5.3 ms with every evaluation in FP64 and the sides
-// doubled up to overflow: about 3000 FP64 evaluations a cone.  The dual cone K* = cl{y3 < 0, -y3 exp(y2/y3) <= e y1}
+// doubled up to overflow (about 3000 FP64 evaluations a cone), 0.45 ms now.  The
+// dual cone K* = cl{y3 < 0, -y3 exp(y2/y3) <= e y1}
 // is projected through Moreau's decomposition, Pi_{K*}(v) = v + Pi_K(-v).
 // ---------------------------------------------------------------------------
 // F for rho <= 0 given e = e^rho, and for rho > 0 given em = e^-rho (scaled by e^-2rho)
@@ -1754,37 +1903,42 @@ static __device__ void expc_project(double& x1, double& x2, double& x3)
     x3 = br;
 }
 
+// Shared memory of a CTA's PSD projections, and where a block's matrices are.
+// Order up to PSD_MAX: X and V, for FP32 also the input matrix and the
+// eigenvectors in FP64 (for the recheck), all in shared memory.  Larger orders:
+// the matrices in the block's global workspace, only the Jacobi scratch in
+// shared memory.
 template <typename T>
 struct PsdSmem {
     T* X;
     T* V;
-    int* pp;
-    int* qq;
-    T* cs;
-    T* sn;
+    T* scratch;   // JacobiScratch (8 bytes a word, for either precision)
     T* lam;
     double* red;
-    double* X0;  // FP32 eigensolves only: the input matrix in FP64 for the residual recheck
+    T* X0;        // FP32 eigensolves only
+    double* V64;
 };
+
+template <typename T>
+__host__ __device__ constexpr size_t psd_small_bytes(int dp)  // matrices of one block of (even) order dp
+{
+    return (size_t)dp * (dp + 1) * (2 * sizeof(T) + (sizeof(T) == 4 ? sizeof(T) + sizeof(double) : 0));
+}
+__host__ __device__ constexpr size_t psd_scratch_bytes(int dp) { return 64 * sizeof(double) + 6 * sizeof(double) * (size_t)dp; }
 
 template <typename T>
 __host__ __device__ constexpr size_t psd_smem_bytes()
 {
-    return sizeof(T) * (2 * PSD_MAX * PSD_LD + 3 * PSD_MAX) + sizeof(int) * PSD_MAX + 64 * sizeof(double) +
-           (sizeof(T) == 4 ? sizeof(double) * PSD_MAX * PSD_LD : 0);
+    return psd_small_bytes<T>(PSD_MAX) + psd_scratch_bytes(PSD_MAX) > psd_scratch_bytes(PSD_BIG_MAX)
+               ? psd_small_bytes<T>(PSD_MAX) + psd_scratch_bytes(PSD_MAX)
+               : psd_scratch_bytes(PSD_BIG_MAX);
 }
 
-// Workspace of one PSD block of order d > PSD_MAX in global memory, with the
-// relative layout of the shared-memory one (X and V adjacent, then cs, sn,
-// lam, pp, qq and, for FP32, X0), so that the FP64 redo's overlays hold:
-// the FP64 eigenvectors over X and V, the FP64 cosines over cs and sn, the
-// FP64 sines over lam.
+// Workspace of one PSD block of order d > PSD_MAX in global memory: the matrices only
 template <typename T>
 __host__ __device__ constexpr size_t psd_big_bytes(int d)
 {
-    const size_t dp = (size_t)(d + (d & 1)), ld = dp + 1;
-    const size_t b = sizeof(T) * (2 * dp * ld + 2 * dp) + sizeof(int) * dp + (sizeof(T) == 4 ? 8 * dp * ld : 0);
-    return (b + 15) & ~size_t(15);
+    return (psd_small_bytes<T>(d + (d & 1)) + 15) & ~size_t(15);
 }
 
 // warm-start eigenvectors of one PSD block: dp x (dp + 1) elements, 16-byte aligned
@@ -1795,36 +1949,21 @@ __host__ __device__ constexpr size_t psd_v_bytes(int d)
     return (sizeof(T) * dp * (dp + 1) + 15) & ~size_t(15);
 }
 
+// smem: the CTA's shared region; big: the block's global workspace, or null
 template <typename T>
-__device__ PsdSmem<T> psd_big_ws(unsigned char* base, int d, double* red)
-{
-    const int dp = d + (d & 1), ld = dp + 1, half = dp / 2;
-    PsdSmem<T> s;
-    s.X = (T*)base;
-    s.V = s.X + (size_t)dp * ld;
-    s.cs = s.V + (size_t)dp * ld;
-    s.sn = s.cs + half;
-    s.lam = s.sn + half;
-    s.red = red;
-    s.pp = (int*)(s.lam + dp);
-    s.qq = s.pp + half;
-    s.X0 = sizeof(T) == 4 ? (double*)(s.qq + half) : nullptr;
-    return s;
-}
-
-template <typename T>
-__device__ PsdSmem<T> psd_smem(unsigned char* base)
+__device__ PsdSmem<T> psd_layout(unsigned char* smem, unsigned char* big, int dp)
 {
     PsdSmem<T> s;
-    s.X = (T*)base;
-    s.V = s.X + PSD_MAX * PSD_LD;
-    s.cs = s.V + PSD_MAX * PSD_LD;
-    s.sn = s.cs + PSD_MAX / 2;
-    s.lam = s.sn + PSD_MAX / 2;
-    s.red = (double*)(s.lam + 2 * PSD_MAX);
-    s.pp = (int*)(s.red + 32);
-    s.qq = s.pp + PSD_MAX / 2;
-    s.X0 = sizeof(T) == 4 ? (double*)(s.qq + PSD_MAX / 2) : nullptr;
+    s.red = (double*)smem;
+    s.scratch = (T*)(s.red + 64);
+    s.lam = (T*)(s.red + 64 + 5 * dp);
+    double* m = big ? (double*)big : s.red + 64 + 6 * dp;
+    const size_t sz = (size_t)dp * (dp + 1);
+    s.V64 = m;
+    if (sizeof(T) == 4) m += sz;
+    s.X = (T*)m;  // 8-byte aligned, and V after it: the FP64 redo's matrix takes the place of both
+    s.V = s.X + sz;
+    s.X0 = s.V + sz;
     return s;
 }
 
@@ -1843,18 +1982,38 @@ struct PsdCheck {
     int* vok;
 };
 
-// FP64 Jacobi of the block whose FP64 copy X0 is in shared memory (FP32
-// eigensolves only).  The FP32 X and V are dead by now: the FP64
-// eigenvectors overlay them (2 PSD_MAX x PSD_LD floats = PSD_MAX x PSD_LD
-// doubles), the rotation cosines and sines the FP32 cs / sn and lam arrays.
-// X0 leaves with the eigenvalues on its diagonal, V64 with the eigenvectors.
-static __device__ __noinline__ void psd_redo_fp64(PsdSmem<float>& sm, int dp, int ld)
+// FP64 Jacobi of the input block X0 (FP32 eigensolves only), in the place of
+// the FP32 X and V, which are dead: that matrix (returned) leaves with the
+// eigenvalues on its diagonal, V64 with the eigenvectors.
+static __device__ __noinline__ double* psd_redo_fp64(PsdSmem<float>& sm, int dp, int ld)
 {
-    double* V64 = reinterpret_cast<double*>(sm.X);
-    double* cs64 = reinterpret_cast<double*>(sm.cs);
-    double* sn64 = reinterpret_cast<double*>(sm.lam);
+    double* X64 = reinterpret_cast<double*>(sm.X);
     __syncthreads();
-    jacobi_block<double>(sm.X0, V64, dp, ld, sm.pp, sm.qq, cs64, sn64, sm.red, 1e-26, 20);
+    for (int i = threadIdx.x; i < dp * ld; i += blockDim.x) X64[i] = (double)sm.X0[i];
+    __syncthreads();
+    jacobi_block<double>(X64, sm.V64, dp, ld, reinterpret_cast<double*>(sm.scratch), sm.red, 1e-26, 20);
+    return X64;
+}
+
+// (V W V^T)(i, j) for i >= j, W = diag(l), from V and U = V W (row stride ld): every entry of
+// the lower triangle by one thread, four rows of a column together; columns with W = 0 skipped.
+template <typename T, class Emit>
+__device__ __forceinline__ void psd_rebuild(const T* U, const T* V, const T* l, int d, int dp, int ld, Emit emit)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i0 = 4 * warp; i0 < d; i0 += 4 * nw)
+        for (int j = lane; j < min(i0 + 4, d); j += 32) {
+            T a[4] = {0, 0, 0, 0};
+            for (int k = 0; k < dp; ++k) {
+                if (l[k] == T(0)) continue;
+                const T v = V[j * ld + k];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) a[h] = fmaT(U[min(i0 + h, d - 1) * ld + k], v, a[h]);
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                if (i0 + h < d && j <= i0 + h) emit(i0 + h, j, a[h]);
+        }
 }
 
 template <typename T, class Team, class Op>
@@ -1911,33 +2070,36 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
     // PSD blocks: one CTA per block, Jacobi eigen-decomposition in shared memory
     // (orders above PSD_MAX: in the block's workspace in global memory)
     if (P.ns > 0) {
-        const PsdSmem<T> sm_small = psd_smem<T>(psd_base);
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
         for (int k = tm.block(); k < P.ns; k += tm.nblocks()) {
             const int d = ro(P.s_dim + k);
             const int o = n + ro(P.s_off + k);
             const int dp = d + (d & 1);
             const int ld = dp + 1;  // odd row stride: column walks are free of bank conflicts
-            PsdSmem<T> sm = d > PSD_MAX ? psd_big_ws<T>(P.psd_big + ro(P.big_off + k), d, sm_small.red) : sm_small;
+            PsdSmem<T> sm = psd_layout<T>(psd_base, d > PSD_MAX ? P.psd_big + ro(P.big_off + k) : nullptr, dp);
             const double isq2 = 0.70710678118654752440;
             __syncthreads();
-            for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x) {
-                const int i = idx / dp, j = idx % dp;
-                T val = 0;
-                if (i < d && j < d) {
-                    const int ii = i > j ? i : j, jj = i > j ? j : i;
-                    T w, wt;
-                    op.load(o + svec_index(d, ii, jj), w, wt);
-                    const T v = T(2) * wt - w;
-                    val = (ii == jj) ? v : (T)((double)v * isq2);
+            for (int j = warp; j < dp; j += nwb)  // column j of the lower triangle: consecutive in svec
+                for (int i = j + lane; i < dp; i += 32) {
+                    T val = 0;
+                    if (i < d) {
+                        T w, wt;
+                        op.load(o + svec_index(d, i, j), w, wt);
+                        const T v = T(2) * wt - w;
+                        val = i == j ? v : (T)((double)v * isq2);
+                    }
+                    sm.X[i * ld + j] = val;
+                    sm.X[j * ld + i] = val;
+                    if constexpr (sizeof(T) == 4) {
+                        sm.X0[i * ld + j] = val;
+                        sm.X0[j * ld + i] = val;
+                    }
                 }
-                sm.X[i * ld + j] = val;
-                if constexpr (sizeof(T) == 4) sm.X0[i * ld + j] = (double)val;
-            }
             __syncthreads();
             const double tol2 = sizeof(T) == 8 ? 1e-26 : 1e-11;
             // Warm start: successive projections of a block see nearby matrices, so the
             // eigenvectors Vp of the last converged decomposition nearly diagonalise this one.
-            // X <- Vp^T X Vp (symmetrised) and V <- Vp, then the sweeps accumulate onto V:
+            // X <- Vp^T X Vp (its lower triangle) and V <- Vp, then the sweeps accumulate onto V:
             // the same eigenpairs, found in a few sweeps instead of a dozen.  vok[k] counts the
             // generations since the last cold start; V loses orthogonality by a few roundings
             // per generation, so every PSD_WARM_GEN-th decomposition starts cold again.
@@ -1946,49 +2108,73 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
             const int gen = Vp ? *(volatile const int*)(ck.vok + k) : 0;
             const bool warm = gen > 0 && gen < PSD_WARM_GEN;
             if (warm) {
-                for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x) {  // V <- X Vp
-                    const int i = idx / dp, j = idx % dp;
-                    T s = 0;
-                    for (int l = 0; l < dp; ++l) s = fmaT(sm.X[i * ld + l], Vp[l * ld + j], s);
-                    sm.V[i * ld + j] = s;
-                }
-                __syncthreads();
-                for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x) {  // X <- Vp^T V
-                    const int i = idx / dp, j = idx % dp;
-                    T s = 0;
-                    for (int l = 0; l < dp; ++l) s = fmaT(Vp[l * ld + i], sm.V[l * ld + j], s);
-                    sm.X[i * ld + j] = s;
-                }
-                __syncthreads();
-                for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x) {
-                    const int i = idx / dp, j = idx % dp;
-                    if (i < j) {
-                        const T a = T(0.5) * (sm.X[i * ld + j] + sm.X[j * ld + i]);
-                        sm.X[i * ld + j] = a;
-                        sm.X[j * ld + i] = a;
+                for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // V <- X Vp, four rows a thread
+                    for (int j = lane; j < dp; j += 32) {
+                        T a[4] = {0, 0, 0, 0};
+                        for (int l = 0; l < dp; ++l) {
+                            const T v = Vp[l * ld + j];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) a[h] = fmaT(sm.X[min(i0 + h, dp - 1) * ld + l], v, a[h]);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            if (i0 + h < dp) sm.V[(i0 + h) * ld + j] = a[h];
                     }
-                    sm.V[i * ld + j] = Vp[i * ld + j];
-                }
+                __syncthreads();
+                for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // X <- Vp^T V, lower triangle
+                    for (int j = lane; j < min(i0 + 4, dp); j += 32) {
+                        T a[4] = {0, 0, 0, 0};
+                        for (int l = 0; l < dp; ++l) {
+                            const T v = sm.V[l * ld + j];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) a[h] = fmaT(Vp[l * ld + min(i0 + h, dp - 1)], v, a[h]);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            if (i0 + h < dp && j <= i0 + h) sm.X[(i0 + h) * ld + j] = a[h];
+                    }
+                __syncthreads();
+                for (int i = warp; i < dp; i += nwb)
+                    for (int j = lane; j < dp; j += 32) sm.V[i * ld + j] = Vp[i * ld + j];
                 __syncthreads();
             }
-            const bool conv = jacobi_block<T>(sm.X, sm.V, dp, ld, sm.pp, sm.qq, sm.cs, sm.sn, sm.red, tol2,
+            const bool conv = jacobi_block<T>(sm.X, sm.V, dp, ld, sm.scratch, sm.red, tol2,
                                               d > PSD_MAX ? 30 : (sizeof(T) == 8 ? 20 : 15), warm);
             if (Vp) {
                 if (conv)
-                    for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x)
-                        Vp[(idx / dp) * ld + idx % dp] = sm.V[(idx / dp) * ld + idx % dp];
+                    for (int i = warp; i < dp; i += nwb)
+                        for (int j = lane; j < dp; j += 32) Vp[i * ld + j] = sm.V[i * ld + j];
                 if (threadIdx.x == 0) ck.vok[k] = conv ? (warm ? gen + 1 : 1) : 0;
+            }
+            for (int i = threadIdx.x; i < dp; i += blockDim.x) {
+                const T l = sm.X[i * ld + i];
+                sm.lam[i] = l > T(0) ? l : T(0);
             }
             if constexpr (sizeof(T) == 4) {
                 // FP64 recheck of the FP32 eigenpairs: ||X V - V diag(l)||_F / ||X||_F
+                for (int i = warp; i < dp; i += nwb)
+                    for (int j = lane; j < dp; j += 32) sm.V64[i * ld + j] = (double)sm.V[i * ld + j];
+                __syncthreads();
                 double r2 = 0.0, x2 = 0.0;
-                for (int idx = threadIdx.x; idx < dp * dp; idx += blockDim.x) {
-                    const int i = idx / dp, k = idx % dp;
-                    double acc = -(double)sm.V[i * ld + k] * (double)sm.X[k * ld + k];
-                    for (int j = 0; j < dp; ++j) acc += sm.X0[i * ld + j] * (double)sm.V[j * ld + k];
-                    r2 += acc * acc;
-                    x2 += sm.X0[i * ld + k] * sm.X0[i * ld + k];
-                }
+                // a warp takes two rows of X0: each lane widens its entries once and hands them round,
+                // so the FP64 pipe does the d^3 multiply-adds and d^2 conversions only
+                for (int i0 = 2 * warp; i0 < dp; i0 += 2 * nwb)
+                    for (int k0 = 0; k0 < dp; k0 += 32) {
+                        const int kk = min(k0 + lane, dp - 1);
+                        const double lk = (double)sm.X[kk * ld + kk];
+                        double a0 = -sm.V64[i0 * ld + kk] * lk, a1 = -sm.V64[(i0 + 1) * ld + kk] * lk;
+                        for (int j0 = 0; j0 < dp; j0 += 32) {
+                            const int jl = min(j0 + lane, dp - 1), jn = min(32, dp - j0);
+                            const double x0 = (double)sm.X0[i0 * ld + jl], x1 = (double)sm.X0[(i0 + 1) * ld + jl];
+                            if (k0 == 0 && lane < jn) x2 += x0 * x0 + x1 * x1;
+                            for (int j = 0; j < jn; ++j) {
+                                const double v = sm.V64[(j0 + j) * ld + kk];
+                                a0 += __shfl_sync(FULL_MASK, x0, j) * v;
+                                a1 += __shfl_sync(FULL_MASK, x1, j) * v;
+                            }
+                        }
+                        if (k0 + lane < dp) r2 += a0 * a0 + a1 * a1;
+                    }
                 r2 = block_sum(r2, sm.red);
                 x2 = block_sum(x2, sm.red);
                 // block_sum hands every thread the same sums, so the decision
@@ -1997,44 +2183,40 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                 if (threadIdx.x == 0 && ck.resid)
                     atomicMax((unsigned long long*)ck.resid, (unsigned long long)__double_as_longlong(rel));
                 if (rel > ck.tol && ck.redo) {
-                    psd_redo_fp64(sm, dp, ld);
+                    double* X64 = psd_redo_fp64(sm, dp, ld);
                     if (threadIdx.x == 0) {
                         atomicAdd((unsigned long long*)ck.redo, 1ull);
                         if (Vp) ck.vok[k] = 0;  // the FP32 eigenvectors were not good enough to start from
                     }
-                    const double* V64 = reinterpret_cast<const double*>(sm.X);
-                    for (int idx = threadIdx.x; idx < d * d; idx += blockDim.x) {
-                        const int i = idx / d, j = idx % d;
-                        if (i < j) continue;
-                        double s = 0.0;
-                        for (int kk = 0; kk < dp; ++kk) {
-                            const double l = sm.X0[kk * ld + kk];
-                            if (l > 0.0) s += V64[i * ld + kk] * l * V64[j * ld + kk];
-                        }
+                    double* lam64 = reinterpret_cast<double*>(sm.scratch);  // the sweeps are over
+                    for (int i = threadIdx.x; i < dp; i += blockDim.x) {
+                        const double l = X64[i * ld + i];
+                        lam64[i] = l > 0.0 ? l : 0.0;
+                    }
+                    __syncthreads();
+                    for (int i = warp; i < dp; i += nwb)
+                        for (int j = lane; j < dp; j += 32) X64[i * ld + j] = sm.V64[i * ld + j] * lam64[j];
+                    __syncthreads();
+                    psd_rebuild<double>(X64, sm.V64, lam64, d, dp, ld, [&](int i, int j, double x) {
                         const int e = o + svec_index(d, i, j);
                         T w, wt;
                         op.load(e, w, wt);
-                        op.store(e, w, wt, (T)(i == j ? s : s * 1.41421356237309504880));
-                    }
+                        op.store(e, w, wt, (T)(i == j ? x : x * 1.41421356237309504880));
+                    });
                     __syncthreads();
                     continue;
                 }
             }
-            for (int i = threadIdx.x; i < dp; i += blockDim.x) {
-                const T l = sm.X[i * ld + i];
-                sm.lam[i] = l > T(0) ? l : T(0);
-            }
             __syncthreads();
-            for (int idx = threadIdx.x; idx < d * d; idx += blockDim.x) {
-                const int i = idx / d, j = idx % d;
-                if (i < j) continue;
-                T s = 0;
-                for (int kk = 0; kk < dp; ++kk) s += sm.V[i * ld + kk] * sm.lam[kk] * sm.V[j * ld + kk];
+            for (int i = warp; i < dp; i += nwb)  // X is dead: V diag(lam) in its place
+                for (int j = lane; j < dp; j += 32) sm.X[i * ld + j] = sm.V[i * ld + j] * sm.lam[j];
+            __syncthreads();
+            psd_rebuild<T>(sm.X, sm.V, sm.lam, d, dp, ld, [&](int i, int j, T x) {
                 const int e = o + svec_index(d, i, j);
                 T w, wt;
                 op.load(e, w, wt);
-                op.store(e, w, wt, i == j ? s : (T)((double)s * 1.41421356237309504880));
-            }
+                op.store(e, w, wt, i == j ? x : (T)((double)x * 1.41421356237309504880));
+            });
             __syncthreads();
         }
     }
