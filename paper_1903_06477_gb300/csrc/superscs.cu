@@ -809,13 +809,19 @@ static size_t dyn_smem(const HostProb& H, int threads, bool tma)
     return std::max(psd, stage);
 }
 
+// Allow the kernels all the dynamic shared memory a block can have.  The limit belongs to the
+// function, not to a work: set to one work's need, it refused the launches of a work with a larger
+// need that had been set up before.
 template <typename T>
-static int config_kernels(size_t dyn, char* err)
+static int config_kernels(char* err)
 {
-    if (dyn > 48 * 1024) {
-        CU(cudaFuncSetAttribute(kgrid_ptr<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn), err);
-        for (const void* fn : {kblock_build<T, BLOCK_SMALL>(), kblock_build<T, BLOCK_LARGE>()})
-            CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn), err);
+    int dev = 0, optin = 0;
+    CU(cudaGetDevice(&dev), err);
+    CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), err);
+    for (const void* fn : {kgrid_ptr<T>(), kblock_build<T, BLOCK_SMALL>(), kblock_build<T, BLOCK_LARGE>()}) {
+        cudaFuncAttributes fa{};
+        CU(cudaFuncGetAttributes(&fa, fn), err);
+        CU(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes), err);
     }
     return SCS_OK;
 }
@@ -1045,8 +1051,8 @@ extern "C" int scs_setup(const scs_data* data, const scs_cone* cone, const scs_s
     w->D.dyn32 = w->has32 ? std::max({dyn_smem<float>(H, w->D.threads, tma), H.cA32.dyn(), H.cAT32.dyn()}) : 0;
     // the FP64 phase of SCS_MIXED also runs FP32 products (refinement corrections)
     if (w->has32) w->D.dyn64 = std::max(w->D.dyn64, w->D.dyn32);
-    int rc2 = config_kernels<double>(w->D.dyn64, w->err);
-    if (!rc2 && w->has32) rc2 = config_kernels<float>(w->D.dyn32, w->err);
+    int rc2 = config_kernels<double>(w->err);
+    if (!rc2 && w->has32) rc2 = config_kernels<float>(w->err);
     if (rc2) { memcpy(g_err, w->err, 512); delete w; return rc2; }
     if (team == SCS_TEAM_GRID) {
         int nb64 = 0, nb32 = 0;
@@ -1604,7 +1610,7 @@ static int batch_finish_setup(scs_batch* b, const scs_settings* settings, scs_ba
     b->dyn64 = any_psd ? psd_smem_bytes<double>() : 0;
     b->dyn32 = any_psd && b->has32 ? psd_smem_bytes<float>() : 0;
     if (b->has32) b->dyn64 = std::max(b->dyn64, b->dyn32);
-    if ((rc = config_kernels<double>(b->dyn64, b->err)) || (b->has32 && (rc = config_kernels<float>(b->dyn32, b->err)))) {
+    if ((rc = config_kernels<double>(b->err)) || (b->has32 && (rc = config_kernels<float>(b->err)))) {
         memcpy(g_err, b->err, 512);
         delete b;
         return rc;
