@@ -1453,6 +1453,8 @@ __device__ __forceinline__ int svec_index(int d, int i, int j)  // i >= j
     return j * d - j * (j - 1) / 2 + (i - j);
 }
 
+// the sum of x over the CTA, in every thread; red: 33 doubles of shared memory.  The warps' sums are
+// added by one warp: every thread adding them itself kept the FP64 pipe busy for 4000 cycles.
 __device__ __forceinline__ double block_sum(double x, double* red)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1460,31 +1462,32 @@ __device__ __forceinline__ double block_sum(double x, double* red)
     __syncthreads();
     if (lane == 0) red[wid] = x;
     __syncthreads();
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += red[w];
+    if (wid == 0) {
+        const double s = warp_sum(lane < nw ? red[lane] : 0.0);
+        if (lane == 0) red[32] = s;
+    }
     __syncthreads();
-    return s;
+    return red[32];
 }
 
 // Parallel two-sided Jacobi (round-robin pairing, dp/2 disjoint rotations per
-// round) on the symmetric dp x dp matrix X (its lower triangle, row stride ld =
-// dp + 1, odd, so that a warp walking a column touches 32 banks); V receives
-// the eigenvectors as columns.  v_init: V already holds an orthogonal start
-// basis (the rotations are accumulated onto it), else it starts as the
-// identity.  Returns true if the off-diagonal mass fell below tol2 times the
-// total within max_sweeps (the same value in every thread); X's diagonal then
-// holds the eigenvalues.
+// round) on a symmetric dp x dp matrix.
 //
-// One CTA barrier a round: the pairs of a round cut X into 2 x 2 blocks (pair
-// k's rows, pair l's columns), each updated from both sides by one thread, and
-// the block that holds the next round's pair k also computes that pair's
-// rotation once it is updated, into the other of two rotation buffers.  (The
-// pairs of round r+1 are (r+1+k, r+1-k), whose members lie in pairs k+1 and
-// k-1 of round r.)  With separate passes for rotations, columns and rows a
-// round took three barriers and updated both triangles: four projections of 512
-// FP32 blocks of order 64 10.0 ms, now 6.5 ms; six FP64 iterations with 150
-// blocks of order 20 to 63 32.6 ms, now 20.8 ms; four with one block of order
-// 120 129 ms, now 76 ms.
+// Round r pairs index r + k with r - k (mod dp - 1; pair 0: r with dp - 1).
+// The matrix is stored by pairs, not by indices: "slot" 2k / 2k+1 is the first
+// / second member of pair k, and a "cell" (k, l), k > l, holds the four values
+// of pair k's rows and pair l's columns, updated from both sides by one thread.
+// The pairs of round r+1 are those of round r with every member moved one slot
+// on (next_slot), the same move in every round, so a thread reads its cell
+// from one buffer and writes the four values to their places of the next round
+// in the other, at addresses that never change; consecutive threads touch
+// consecutive words.  The cells (k+1, k-1) hold the next round's pair k: their
+// threads also compute its rotation, straight from the register.  So a round
+// takes one CTA barrier and no index arithmetic.  (Three passes over an indexed
+// matrix with a barrier each: 4400 cycles a round for order 64 in FP32, 12000 in
+// FP64; one pass over the indexed lower triangle: 2400 and 10800; the cells: 1160
+// and 6540.  512 blocks of order 64 in FP32, one projection: 10.0, 6.5 and 4.6 ms;
+// one block of order 120 in FP64, four iterations: 129, 76 and 42 ms.)
 //
 // FP64: the FP64 pipe (2 multiply-adds a cycle and SM) is the bound, so the
 // rotations are applied in scaled form (fast Givens): X = D X^ D and V = V^ D
@@ -1493,126 +1496,186 @@ __device__ __forceinline__ double block_sum(double x, double* red)
 // after each sweep (its entries shrink by at most sqrt(2) a round).  The angle
 // is found in FP32 -- any t with c = 1/sqrt(1 + t^2), s = t c is a rotation,
 // and c, the scales and the diagonal are FP64 for the t that was taken; an
-// angle 1e-7 off leaves 1e-7 of the element for the next sweep.  Per round
-// dp^2 + dp^2 / 2 multiply-adds against 3 dp^2 products and multiply-adds.
+// angle 1e-7 off leaves 1e-7 of the element for the next sweep.
+//
+// V (columns contiguous, stride ldv) receives the eigenvectors; its update is
+// left to the warps that compute no rotations, a round's longest chain.
 template <typename T>
-struct JacobiScratch {
-    T *r0, *r1;         // rotations of a round, two buffers of dp/2: (c, s), or (al, be) in FP64
-    T *dg, *sc, *isc;   // FP64: the diagonal of X, the scales D and 1 / D (dp each)
-    static constexpr int words(int dp) { return 5 * dp; }
-    __device__ JacobiScratch(T* base, int dp) : r0(base), r1(base + dp), dg(base + 2 * dp), sc(base + 3 * dp), isc(base + 4 * dp) {}
+struct Jacobi {
+    T* cell[2];   // two buffers of 4 x ncell values: component c of cell i at c * ncell + i
+    T* V;
+    T* rot;       // [2][dp/2][2]: rotations of a round, (c, s), or (al, be) in FP64
+    T* dg;        // [2][dp]: the diagonal by slots
+    T *sc, *isc;  // FP64: [2][dp], the scales D and 1 / D by slots
+    T *e, *def;   // dp/2 each: the pairs' own off-diagonal values at a sweep's start; after their rotation
+    int dp, half, ncell, ldv;
+    static constexpr int scratch_words(int dp) { return 9 * dp; }
+    __host__ __device__ static constexpr int cells(int dp) { return (dp / 2) * (dp / 2 - 1) / 2; }
+    __device__ Jacobi(T* c0, T* c1, T* v, T* scratch, int dp_, int ldv_)
+        : V(v), rot(scratch), dg(scratch + 2 * dp_), sc(scratch + 4 * dp_), isc(scratch + 6 * dp_), e(scratch + 8 * dp_),
+          def(e + dp_ / 2), dp(dp_), half(dp_ / 2), ncell(cells(dp_)), ldv(ldv_)
+    {
+        cell[0] = c0;
+        cell[1] = c1;
+    }
+    __device__ __forceinline__ int slot_of(int i) const  // of index i at a sweep's start
+    {
+        return i == dp - 1 ? 1 : (i < half ? 2 * i : 2 * (dp - 1 - i) + 1);
+    }
+    // offset of the value at slots (a, b) of two different pairs
+    __device__ __forceinline__ int at(int a, int b) const
+    {
+        const int k = a >> 1, l = b >> 1;
+        return k > l ? ((a & 1) * 2 + (b & 1)) * ncell + k * (k - 1) / 2 + l
+                     : ((b & 1) * 2 + (a & 1)) * ncell + l * (l - 1) / 2 + k;
+    }
+    // the slot of the next round
+    __device__ __forceinline__ int next_slot(int a) const
+    {
+        const int k = a >> 1;
+        if (a & 1) return k == 0 ? 1 : (k == half - 1 ? a - 1 : a + 2);
+        return k == 0 ? 3 : a - 2;
+    }
+    // entry (i, j) of the matrix at the start (any i, j of the lower triangle, once each)
+    __device__ __forceinline__ void put(int i, int j, T x) const
+    {
+        const int a = slot_of(i), b = slot_of(j);
+        if (i == j)
+            dg[a] = x;
+        else if ((a >> 1) == (b >> 1))
+            e[a >> 1] = x;
+        else
+            cell[0][at(a, b)] = x;
+    }
 };
 
-// block idx of a round (half >= 3): the first `half` hold next round's pairs, see jacobi_block
-__device__ __forceinline__ void jacobi_cell(int idx, int half, int& k, int& l)
+// tan of the rotation that annihilates apq, the smaller root of t^2 + 2 th t - 1
+// = 0 with th = diff / (2 apq), by the hardware's approximate reciprocal and
+// square root: it is on the round's critical path, and any t is a rotation.
+__device__ __forceinline__ float jacobi_tan(float diff, float apq)
 {
-    if (idx < half) {
-        k = min(idx + 1, half - 1);
-        l = idx == half - 1 ? half - 2 : max(idx - 1, 0);
-        return;
-    }
-    idx -= half;
-    if (idx < half - 3) {  // neighbours (k - l = 1) but the first and the last
-        k = idx + 2;
-        l = idx + 1;
-        return;
-    }
-    idx -= half - 3;  // k - l >= 3: a triangle
-    int r = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
-    while ((r + 1) * (r + 2) / 2 <= idx) ++r;
-    while (r * (r + 1) / 2 > idx) --r;
-    k = r + 3;
-    l = idx - r * (r + 1) / 2;
+    if (apq == 0.f) return 0.f;
+    const float th = __fdividef(0.5f * diff, apq), at = fabsf(th);
+    if (!(at < 1e18f)) return at < 1e38f ? __fdividef(0.5f, th) : 0.f;
+    float root;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(th, th, 1.f)));
+    return copysignf(__fdividef(1.f, at + root), th);
 }
 
+// Sweeps until the off-diagonal mass is below tol2 times the total, at most
+// max_sweeps (FP32: V is updated only, so it must hold the start basis; the
+// matrix has been put).  Returns whether it is (the same value in every
+// thread); dg[slot_of(i)] of buffer `cur` then is eigenvalue i.
 template <typename T>
-__device__ bool jacobi_block(T* X, T* V, int dp, int ld, T* scratch, double* red, double tol2, int max_sweeps,
-                             bool v_init = false)
+__device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int max_sweeps, int& cur)
 {
     constexpr bool kFast = sizeof(T) == 8;
-    const JacobiScratch<T> S(scratch, dp);
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    const int half = dp / 2, ncell = half * (half - 1) / 2;
-    double total = 0.0;
-    for (int i = warp; i < dp; i += nw) {
-        for (int j = lane; j < i; j += 32) total += 2.0 * (double)X[i * ld + j] * (double)X[i * ld + j];
-        if (lane == 0) total += (double)X[i * ld + i] * (double)X[i * ld + i];
-        if (!v_init)
-            for (int j = lane; j < dp; j += 32) V[i * ld + j] = (i == j) ? T(1) : T(0);
-    }
-    if constexpr (kFast)
-        for (int i = tid; i < dp; i += nt) {
-            S.dg[i] = X[i * ld + i];
-            S.sc[i] = S.isc[i] = T(1);
-        }
-    total = block_sum(total, red);
-    // FP64: a power of two that brings the matrix to about 1, for the FP32 angles
-    const double unit = kFast && total > 0.0 && isfinite(total) ? scalbn(1.0, -ilogb(sqrt(total))) : 1.0;
-    auto pair = [&](int k, int rnd, int& p, int& q) {  // pair k of a round, p < q
-        int a = rnd, b = dp - 1;
-        if (k > 0) {
-            a = rnd + k;
-            if (a >= dp - 1) a -= dp - 1;
-            b = rnd - k;
-            if (b < 0) b += dp - 1;
-        }
-        p = min(a, b);
-        q = max(a, b);
+    constexpr int VW = 16 / (int)sizeof(T);  // rows of V a thread moves at a time
+    constexpr int NC = 3;                    // cells of a thread, besides the owned one, whose addresses are kept
+    const int tid = threadIdx.x, nt = blockDim.x, nw = nt >> 5;
+    const int dp = J.dp, half = J.half, ncell = J.ncell;
+    struct Cell {
+        int k, l, src, dst[4];
     };
-    auto at = [&](int i, int j) { return i > j ? i * ld + j : j * ld + i; };
-    // the rotation of pair k of a round into buffer buf, applied to the pair's own 2 x 2 block
-    auto rotate = [&](int k, int rnd, int buf) {
-        int p, q;
-        pair(k, rnd, p, q);
+    auto make_cell = [&](int idx) {
+        Cell c;
+        if (idx < half) {  // the cells that hold next round's pairs
+            c.k = min(idx + 1, half - 1);
+            c.l = idx == half - 1 ? half - 2 : max(idx - 1, 0);
+        } else if (idx < 2 * half - 3) {  // neighbours (k - l = 1) but the first and the last
+            c.k = idx - half + 2;
+            c.l = c.k - 1;
+        } else {  // k - l >= 3: a triangle
+            const int i = idx - (2 * half - 3);
+            int r = (int)((sqrtf(8.0f * (float)i + 1.0f) - 1.0f) * 0.5f);
+            while ((r + 1) * (r + 2) / 2 <= i) ++r;
+            while (r * (r + 1) / 2 > i) --r;
+            c.k = r + 3;
+            c.l = i - r * (r + 1) / 2;
+        }
+        c.src = c.k * (c.k - 1) / 2 + c.l;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int a = J.next_slot(2 * c.k + (q >> 1)), b = J.next_slot(2 * c.l + (q & 1));
+            c.dst[q] = (a >> 1) == (b >> 1) ? -1 : J.at(a, b);
+        }
+        return c;
+    };
+    // Roles: the first `own` warps have the cells that hold the next round's pairs and their rotations,
+    // a round's longest chain; the other cells and V go to the other warps, where there are any.
+    const int own = (half + 31) >> 5;
+    const bool split = nw > own;
+    const int ostep = split ? 32 * own : nt, vt0 = split ? 32 * own : 0, vn = nt - vt0, vtid = tid - vt0;
+    const bool owner = tid < ostep && half >= 3;
+    Cell mine{}, kept[NC];
+    if (owner && tid < half) mine = make_cell(tid);
+#pragma unroll
+    for (int n = 0; n < NC; ++n)
+        if (vtid >= 0 && half + vtid + n * vn < ncell) kept[n] = make_cell(half + vtid + n * vn);
+    T* const buf0 = J.cell[0];  // (an indexed J.cell would live in local memory)
+    T* const buf1 = J.cell[1];
+    // a pair's members' slots in the round before, and where its own value goes in the next
+    auto from_a = [&](int k) { return k < half - 1 ? 2 * k + 2 : 2 * half - 1; };
+    auto from_b = [&](int k) { return k == 0 ? 1 : (k == 1 ? 0 : 2 * k - 1); };
+    auto def_to = [&](int k) { return J.at(J.next_slot(2 * k), J.next_slot(2 * k + 1)); };
+    const int my_a = from_a(tid), my_b = from_b(tid), my_def = owner && tid < half ? def_to(tid) : 0;
+    // what a rotation needs of the round before: loaded ahead of the cell that holds its value
+    struct Own {
+        T app, aqq, sp, sq, ep, eq;
+    };
+    auto ahead = [&](int fr, int a, int b) {
+        Own o;
+        o.app = J.dg[fr * dp + a];
+        o.aqq = J.dg[fr * dp + b];
         if constexpr (kFast) {
-            const T dp_ = S.sc[p], dq = S.sc[q], ep = S.isc[p], eq = S.isc[q], app = S.dg[p], aqq = S.dg[q];
-            const T apq = X[q * ld + p] * (dp_ * dq), diff = aqq - app;
-            const float den = (float)(apq * unit), num = (float)(diff * unit);
-            float tf = 0.f;
-            if (den != 0.f) {
-                const float th = num / (2.f * den), at_ = fabsf(th);
-                tf = at_ > 1e18f ? 0.5f / th : copysignf(1.f, th) / (at_ + sqrtf(th * th + 1.f));
-            }
-            const T t = (T)tf, a = fma(t, t, T(1));
-            T c = (T)rsqrtf((float)a);  // two Newton steps to 1 / sqrt(1 + t^2)
-            c = c * fma(T(-0.5) * a * c, c, T(1.5));
-            c = c * fma(T(-0.5) * a * c, c, T(1.5));
-            const T ic = a * c, h = c * c;
-            const T del = h * t * (t * diff - T(2) * apq);
-            S.r0[buf * half + k] = t * dq * ep;
-            S.r1[buf * half + k] = t * dp_ * eq;
-            S.dg[p] = app + del;
-            S.dg[q] = aqq - del;
-            S.sc[p] = c * dp_;
-            S.sc[q] = c * dq;
-            S.isc[p] = ic * ep;
-            S.isc[q] = ic * eq;
-            X[q * ld + p] = h * (fma(-t, t, T(1)) * apq - t * diff) * (ic * ep) * (ic * eq);
+            o.sp = J.sc[fr * dp + a];
+            o.sq = J.sc[fr * dp + b];
+            o.ep = J.isc[fr * dp + a];
+            o.eq = J.isc[fr * dp + b];
+        }
+        return o;
+    };
+    // rotation of pair k, whose off-diagonal value is x, into buffer `to`
+    auto rotate = [&](int k, T x, const Own& o, int to) {
+        T *dgt = J.dg + to * dp + 2 * k, *sct = J.sc + to * dp + 2 * k, *ist = J.isc + to * dp + 2 * k;
+        T* rt = J.rot + (to * half + k) * 2;
+        const T app = o.app, aqq = o.aqq, diff = aqq - app;
+        if constexpr (kFast) {
+            const T sp = o.sp, sq = o.sq, ep = o.ep, eq = o.eq;
+            const T apq = x * (sp * sq);
+            const float tf = jacobi_tan((float)diff, (float)apq);
+            const T t = (T)tf, al = t * (sq * ep), be = t * (sp * eq);
+            rt[0] = al;
+            rt[1] = be;
+            // the factors c^2 of the rotation and 1 / c^2 of the scales cancel
+            J.def[k] = fma(fma(-t, t, T(1)), apq, -t * diff) * (ep * eq);
+            // c = 1 / sqrt(1 + t^2) from its FP32 value: (1 + d)^-1/2 to second order in d = 1e-7
+            const T a2 = fma(t, t, T(1)), c0 = (T)rsqrtf(fmaf(tf, tf, 1.f)), d = fma(a2 * c0, c0, T(-1));
+            const T c = c0 * fma(d, fma(d, T(0.375), T(-0.5)), T(1)), ic = a2 * c;
+            const T del = (c * c) * (t * fma(t, diff, T(-2) * apq));
+            dgt[0] = app + del;
+            dgt[1] = aqq - del;
+            sct[0] = c * sp;
+            sct[1] = c * sq;
+            ist[0] = ic * ep;
+            ist[1] = ic * eq;
         } else {
-            const T app = X[p * ld + p], aqq = X[q * ld + q], apq = X[q * ld + p];
-            T c = 1, s = 0;
-            if (apq != T(0)) {
-                const T theta = (aqq - app) / (T(2) * apq);
-                const T at_ = theta < T(0) ? -theta : theta;
-                T t;
-                if (at_ > T(1e18))
-                    t = T(0.5) / theta;
-                else
-                    t = (theta >= T(0) ? T(1) : T(-1)) / (at_ + sqrt(theta * theta + T(1)));
-                c = T(1) / sqrt(t * t + T(1));
-                s = t * c;
-            }
-            S.r0[buf * half + k] = c;
-            S.r1[buf * half + k] = s;
-            const T xpp = c * app - s * apq, xpq = s * app + c * apq;  // columns, then rows
-            const T xqp = c * apq - s * aqq, xqq = s * apq + c * aqq;
-            X[p * ld + p] = c * xpp - s * xqp;
-            X[q * ld + p] = c * xpq - s * xqq;
-            X[q * ld + q] = s * xpq + c * xqq;
+            // c as the quotient of two correctly rounded operations, each by one Newton step from the
+            // hardware's approximation (Markstein, 1990; a in [1, 2]): V's slow loss of
+            // orthogonality depends on how c is rounded, and stays what it was
+            const T t = jacobi_tan(diff, x), a2 = t * t + T(1);
+            const T y = rsqrtf(a2), g0 = a2 * y, g = fmaf(fmaf(-g0, g0, a2), T(0.5) * y, g0);
+            const T c0 = __fdividef(1.f, g), c = fmaf(fmaf(-g, c0, 1.f), c0, c0), s = t * c;
+            rt[0] = c;
+            rt[1] = s;
+            const T xpp = c * app - s * x, xpq = s * app + c * x;  // columns, then rows
+            const T xqp = c * x - s * aqq, xqq = s * x + c * aqq;
+            dgt[0] = c * xpp - s * xqp;
+            J.def[k] = c * xpq - s * xqq;
+            dgt[1] = s * xpq + c * xqq;
         }
     };
-    // (x_p, x_q) through one rotation
-    auto turn = [](T& xp, T& xq, T r0, T r1) {
+    auto turn = [](T& xp, T& xq, T r0, T r1) {  // (x_p, x_q) through one rotation
         const T a = xp, b = xq;
         if constexpr (kFast) {
             xp = fma(-r0, b, a);
@@ -1622,86 +1685,171 @@ __device__ bool jacobi_block(T* X, T* V, int dp, int ld, T* scratch, double* red
             xq = r1 * a + r0 * b;
         }
     };
-    int kc[2] = {0, 0}, lc[2] = {0, 0};  // this thread's first two cells
-    if (half >= 3) {
-        if (tid < ncell) jacobi_cell(tid, half, kc[0], lc[0]);
-        if (tid + nt < ncell) jacobi_cell(tid + nt, half, kc[1], lc[1]);
-    } else {
-        kc[0] = 1;
-    }
-    const bool wide = nt >= dp;  // V: a thread has one row and every ng-th pair, or all pairs of several rows
-    const int vi0 = wide ? tid % dp : tid, vstep = wide ? dp : nt, ng = wide ? nt / dp : 1, vg = wide ? tid / dp : 0;
-    bool conv = false;
-    for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
-        double off = 0.0;
-        for (int i = warp; i < dp; i += nw) {
-            if constexpr (kFast) {
-                const T di = S.sc[i];
-                for (int j = lane; j < i; j += 32) {
-                    const T x = X[i * ld + j] * (di * S.sc[j]);
-                    X[i * ld + j] = x;
-                    off += x * x;
-                }
-                if (sweep > 0)
-                    for (int j = lane; j < dp; j += 32) V[i * ld + j] *= S.sc[j];
-            } else {
-                for (int j = lane; j < i; j += 32) off += (double)X[i * ld + j] * (double)X[i * ld + j];
-            }
+    // the whole matrix is put; its total, and in FP64 a power of four that scales it to about 1 for
+    // the FP32 angles (through the first D)
+    auto square_sum = [&](int buf) {
+        double s = 0.0;
+        const T* c = buf ? buf1 : buf0;
+        for (int i = tid; i < 4 * ncell; i += nt) s += (double)c[i] * (double)c[i];
+        for (int i = tid; i < half; i += nt) s += (double)J.e[i] * (double)J.e[i];
+        return 2.0 * s;
+    };
+    __syncthreads();
+    double total = square_sum(0);
+    for (int i = tid; i < dp; i += nt) total += (double)J.dg[i] * (double)J.dg[i];
+    total = block_sum(total, red);
+    const int quad = kFast && total > 0.0 && isfinite(total) ? ilogb(total) / 4 : 0;
+    if constexpr (kFast) {
+        for (int i = tid; i < dp; i += nt) {
+            J.dg[i] = scalbn(J.dg[i], -2 * quad);
+            J.sc[i] = scalbn(1.0, -quad);
         }
-        off = 2.0 * block_sum(off, red);
-        conv = off <= tol2 * total || off == 0.0;
-        if (conv || sweep == max_sweeps) break;
+        total = scalbn(total, -4 * quad);
+        __syncthreads();
+    }
+    // V: a thread has VW rows and every ng-th pair, or all pairs of several row groups
+    const int groups = J.ldv / VW;
+    const bool wide = vn >= groups;
+    const int vi0 = vtid < 0 ? groups : (wide ? vtid % groups : vtid), vstep = wide ? groups : vn;
+    const int ng = wide ? vn / groups : 1, vg = wide ? vtid / groups : 0;
+    bool conv = false;
+    cur = 0;
+    for (int sweep = 0; sweep <= max_sweeps; ++sweep) {
         if constexpr (kFast) {
-            for (int i = tid; i < dp; i += nt) S.sc[i] = S.isc[i] = T(1);
+            T* c = cur ? buf1 : buf0;
+            const T* sc = J.sc + cur * dp;
+            for (int i = tid; i < ncell; i += nt) {
+                int k = (int)((sqrtf(8.0f * (float)i + 1.0f) + 1.0f) * 0.5f);
+                while (k * (k + 1) / 2 <= i) ++k;
+                while (k * (k - 1) / 2 > i) --k;
+                const int l = i - k * (k - 1) / 2;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) c[q * ncell + i] *= sc[2 * k + (q >> 1)] * sc[2 * l + (q & 1)];
+            }
+            for (int i = tid; i < half; i += nt) J.e[i] *= sc[2 * i] * sc[2 * i + 1];
+            if (sweep > 0)
+                for (int j = tid >> 5; j < dp; j += nw) {
+                    const T f = sc[J.slot_of(j)];
+                    for (int i = tid & 31; i < dp; i += 32) J.V[j * J.ldv + i] *= f;
+                }
             __syncthreads();
         }
-        for (int k = tid; k < half; k += nt) rotate(k, 0, 0);
+        const double off = block_sum(square_sum(cur), red);
+        conv = off <= tol2 * total || off == 0.0;
+        if (conv || sweep == max_sweeps) break;
+        for (int k = tid; k < half; k += nt) {
+            if constexpr (kFast) {
+                J.sc[cur * dp + 2 * k] = J.sc[cur * dp + 2 * k + 1] = T(1);
+                J.isc[cur * dp + 2 * k] = J.isc[cur * dp + 2 * k + 1] = T(1);
+            }
+            rotate(k, J.e[k], ahead(cur, 2 * k, 2 * k + 1), cur);
+        }
         __syncthreads();
         for (int rnd = 0; rnd < dp - 1; ++rnd) {
-            const T* r0 = S.r0 + (rnd & 1) * half;
-            const T* r1 = S.r1 + (rnd & 1) * half;
-            for (int idx = tid, n = 0; idx < ncell; idx += nt, ++n) {
-                int k, l, pk, qk, pl, ql;
-                if (n < 2) {
-                    k = n == 0 ? kc[0] : kc[1];
-                    l = n == 0 ? lc[0] : lc[1];
-                } else {
-                    jacobi_cell(idx, half, k, l);
+            const T* rot = J.rot + cur * dp;
+            const T* src = cur ? buf1 : buf0;
+            T* dst = cur ? buf0 : buf1;
+            const bool last = rnd == dp - 2;
+            // a cell's four values through its two rotations
+            auto load_turn = [&](const Cell& c, T(&x)[4]) {
+                const T ck = rot[2 * c.k], sk = rot[2 * c.k + 1], cl = rot[2 * c.l], sl = rot[2 * c.l + 1];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) x[q] = src[q * ncell + c.src];
+                turn(x[0], x[1], cl, sl);
+                turn(x[2], x[3], cl, sl);
+                turn(x[0], x[2], ck, sk);
+                turn(x[1], x[3], ck, sk);
+            };
+            auto run_cell = [&](const Cell& c) {
+                T x[4];
+                load_turn(c, x);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) dst[c.dst[q]] = x[q];
+            };
+            auto run_owned = [&](const Cell& c, int k, int a, int b, int to_def) {
+                dst[to_def] = J.def[k];  // the pair's own value, rotated before this round
+                const Own o = ahead(cur, a, b);
+                T x[4], v = 0;
+                load_turn(c, x);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    v = c.dst[q] < 0 ? x[q] : v;
+                    if (c.dst[q] >= 0) dst[c.dst[q]] = x[q];
                 }
-                pair(k, rnd, pk, qk);
-                pair(l, rnd, pl, ql);
-                const T ck = r0[k], sk = r1[k], cl = r0[l], sl = r1[l];
-                const int ia = at(pk, pl), ib = at(pk, ql), ic = at(qk, pl), id = at(qk, ql);
-                T xa = X[ia], xb = X[ib], xc = X[ic], xd = X[id];
-                turn(xa, xb, cl, sl);
-                turn(xc, xd, cl, sl);
-                turn(xa, xc, ck, sk);
-                turn(xb, xd, ck, sk);
-                X[ia] = xa;
-                X[ib] = xb;
-                X[ic] = xc;
-                X[id] = xd;
-                if (idx < half && rnd + 1 < dp - 1) {
-                    rotate(idx, rnd + 1, (rnd + 1) & 1);
-                    if (half == 2) rotate(1, rnd + 1, (rnd + 1) & 1);
+                if (last)
+                    J.e[k] = v;
+                else
+                    rotate(k, v, o, cur ^ 1);
+            };
+            if (owner) {
+                if (tid < half) run_owned(mine, tid, my_a, my_b, my_def);
+                for (int k = tid + ostep; k < half; k += ostep)
+                    run_owned(make_cell(k), k, from_a(k), from_b(k), def_to(k));
+            } else if (half < 3 && tid == 0) {
+                if (half == 1) {
+                    J.e[0] = J.def[0];
+                } else {  // one cell, which holds both of the next pairs: (a1, b0) and (b1, a0)
+                    Cell c;
+                    c.k = 1;
+                    c.l = c.src = 0;
+                    T x[4];
+                    load_turn(c, x);
+                    dst[J.at(3, 1)] = J.def[0];
+                    dst[J.at(0, 2)] = J.def[1];
+                    dst[J.at(0, 3)] = x[0];
+                    dst[J.at(2, 1)] = x[3];
+                    if (last) {
+                        J.e[0] = x[1];
+                        J.e[1] = x[2];
+                    } else {
+                        rotate(0, x[1], ahead(cur, from_a(0), from_b(0)), cur ^ 1);
+                        rotate(1, x[2], ahead(cur, from_a(1), from_b(1)), cur ^ 1);
+                    }
                 }
             }
-            for (int i = vi0; i < dp; i += vstep)
-                for (int k = vg; k < half && vg < ng; k += ng) {
-                    int p, q;
-                    pair(k, rnd, p, q);
-                    const T c = r0[k], s = r1[k];
-                    if (kFast && c == T(0) && s == T(0)) continue;
-                    T vp = V[i * ld + p], vq = V[i * ld + q];
-                    turn(vp, vq, c, s);
-                    V[i * ld + p] = vp;
-                    V[i * ld + q] = vq;
+            if (vtid >= 0 && half >= 3) {
+#pragma unroll
+                for (int n = 0; n < NC; ++n)
+                    if (half + vtid + n * vn < ncell) run_cell(kept[n]);
+                for (int idx = half + vtid + NC * vn; idx < ncell; idx += vn) run_cell(make_cell(idx));
+            }
+            if (vg < ng)
+                for (int i = vi0; i < groups; i += vstep) {
+                    struct alignas(16) Vec {
+                        T x[VW];
+                    };
+                    T* Vi = J.V + i * VW;
+                    for (int k = vg; k < half; k += ng) {
+                        const T c = rot[2 * k], sn = rot[2 * k + 1];
+                        int a = rnd, b = dp - 1;
+                        if (k > 0) {
+                            a = rnd + k;
+                            if (a >= dp - 1) a -= dp - 1;
+                            b = rnd - k;
+                            if (b < 0) b += dp - 1;
+                        }
+                        Vec va = *reinterpret_cast<const Vec*>(Vi + a * J.ldv), vb = *reinterpret_cast<const Vec*>(Vi + b * J.ldv);
+#pragma unroll
+                        for (int h = 0; h < VW; ++h) turn(va.x[h], vb.x[h], c, sn);
+                        *reinterpret_cast<Vec*>(Vi + a * J.ldv) = va;
+                        *reinterpret_cast<Vec*>(Vi + b * J.ldv) = vb;
+                    }
+                }
+            cur ^= 1;
+            if (last)  // the diagonal (and the scales) of round dp - 2, by the slots of the next sweep
+                for (int a = tid; a < dp; a += nt) {
+                    const int b = half == 1 ? a : J.next_slot(a);
+                    J.dg[cur * dp + b] = J.dg[(cur ^ 1) * dp + a];
+                    if constexpr (kFast) {
+                        J.sc[cur * dp + b] = J.sc[(cur ^ 1) * dp + a];
+                        J.isc[cur * dp + b] = J.isc[(cur ^ 1) * dp + a];
+                    }
                 }
             __syncthreads();
         }
     }
     if constexpr (kFast) {
-        for (int i = tid; i < dp; i += nt) X[i * ld + i] = S.dg[i];
+        for (int i = tid; i < dp; i += nt) J.dg[cur * dp + i] = scalbn(J.dg[cur * dp + i], 2 * quad);
         __syncthreads();
     }
     return conv;
@@ -1903,50 +2051,52 @@ static __device__ void expc_project(double& x1, double& x2, double& x3)
     x3 = br;
 }
 
-// Shared memory of a CTA's PSD projections, and where a block's matrices are.
-// Order up to PSD_MAX: X and V, for FP32 also the input matrix and the
-// eigenvectors in FP64 (for the recheck), all in shared memory.  Larger orders:
-// the matrices in the block's global workspace, only the Jacobi scratch in
-// shared memory.
+// Shared memory of a CTA's PSD projections, and where a block's matrices are:
+// all in shared memory up to order PSD_MAX; larger orders in the block's global
+// workspace, with the Jacobi scratch in shared memory.
 template <typename T>
 struct PsdSmem {
-    T* X;
-    T* V;
-    T* scratch;   // JacobiScratch (8 bytes a word, for either precision)
+    T* X0;        // the input matrix, full, row stride dp + 1; FP64: later the second cell buffer
+    T* V;         // X Vp while a warm start is formed (row stride dp + 1), then the eigenvectors (columns, stride ldv)
+    T* cell[2];
+    double* V64;  // FP32 eigensolves only: the eigenvectors in FP64 (row stride dp + 1), for the recheck
+    T* scratch;   // Jacobi's scratch, 8 bytes a word in either precision
     T* lam;
     double* red;
-    T* X0;        // FP32 eigensolves only
-    double* V64;
 };
 
+// stride of V's columns: whole 16-byte vectors
 template <typename T>
-__host__ __device__ constexpr size_t psd_small_bytes(int dp)  // matrices of one block of (even) order dp
+__host__ __device__ constexpr int psd_ldv(int dp)
 {
-    return (size_t)dp * (dp + 1) * (2 * sizeof(T) + (sizeof(T) == 4 ? sizeof(T) + sizeof(double) : 0));
+    return sizeof(T) == 4 ? (dp + 3) & ~3 : dp;
 }
-__host__ __device__ constexpr size_t psd_scratch_bytes(int dp) { return 64 * sizeof(double) + 6 * sizeof(double) * (size_t)dp; }
-
+__host__ __device__ constexpr size_t psd_round(size_t bytes) { return (bytes + 15) & ~size_t(15); }
 template <typename T>
-__host__ __device__ constexpr size_t psd_smem_bytes()
+__host__ __device__ constexpr size_t psd_matrix_bytes(int dp)  // matrices of one block of (even) order dp
 {
-    return psd_small_bytes<T>(PSD_MAX) + psd_scratch_bytes(PSD_MAX) > psd_scratch_bytes(PSD_BIG_MAX)
-               ? psd_small_bytes<T>(PSD_MAX) + psd_scratch_bytes(PSD_MAX)
-               : psd_scratch_bytes(PSD_BIG_MAX);
+    return 2 * psd_round(sizeof(T) * (size_t)dp * (dp + 2)) + (sizeof(T) == 4 ? 2 : 1) * psd_round(sizeof(T) * 4 * (size_t)Jacobi<T>::cells(dp)) +
+           (sizeof(T) == 4 ? psd_round(sizeof(double) * (size_t)dp * (dp + 1)) : 0);
 }
-
-// Workspace of one PSD block of order d > PSD_MAX in global memory: the matrices only
+__host__ __device__ constexpr size_t psd_scratch_bytes(int dp) { return sizeof(double) * (64 + 10 * (size_t)dp); }
+// dynamic shared memory of a CTA that projects blocks of order d
+template <typename T>
+__host__ __device__ constexpr size_t psd_smem_bytes(int d)
+{
+    return psd_scratch_bytes(d + (d & 1)) + (d <= PSD_MAX ? psd_matrix_bytes<T>(d + (d & 1)) : 0);
+}
+// workspace of one PSD block of order d > PSD_MAX in global memory
 template <typename T>
 __host__ __device__ constexpr size_t psd_big_bytes(int d)
 {
-    return (psd_small_bytes<T>(d + (d & 1)) + 15) & ~size_t(15);
+    return psd_matrix_bytes<T>(d + (d & 1));
 }
-
-// warm-start eigenvectors of one PSD block: dp x (dp + 1) elements, 16-byte aligned
+// warm-start eigenvectors of one PSD block: dp columns
 template <typename T>
 __host__ __device__ constexpr size_t psd_v_bytes(int d)
 {
-    const size_t dp = (size_t)(d + (d & 1));
-    return (sizeof(T) * dp * (dp + 1) + 15) & ~size_t(15);
+    const int dp = d + (d & 1);
+    return psd_round(sizeof(T) * (size_t)dp * psd_ldv<T>(dp));
 }
 
 // smem: the CTA's shared region; big: the block's global workspace, or null
@@ -1956,14 +2106,16 @@ __device__ PsdSmem<T> psd_layout(unsigned char* smem, unsigned char* big, int dp
     PsdSmem<T> s;
     s.red = (double*)smem;
     s.scratch = (T*)(s.red + 64);
-    s.lam = (T*)(s.red + 64 + 5 * dp);
-    double* m = big ? (double*)big : s.red + 64 + 6 * dp;
-    const size_t sz = (size_t)dp * (dp + 1);
-    s.V64 = m;
-    if (sizeof(T) == 4) m += sz;
-    s.X = (T*)m;  // 8-byte aligned, and V after it: the FP64 redo's matrix takes the place of both
-    s.V = s.X + sz;
-    s.X0 = s.V + sz;
+    s.lam = (T*)(s.red + 64 + 9 * dp);
+    unsigned char* m = big ? big : smem + psd_scratch_bytes(dp);
+    s.V64 = (double*)m;
+    if (sizeof(T) == 4) m += psd_round(sizeof(double) * (size_t)dp * (dp + 1));
+    s.X0 = (T*)m;
+    m += psd_round(sizeof(T) * (size_t)dp * (dp + 2));
+    s.V = (T*)m;
+    m += psd_round(sizeof(T) * (size_t)dp * (dp + 2));
+    s.cell[0] = (T*)m;
+    s.cell[1] = sizeof(T) == 4 ? (T*)(m + psd_round(sizeof(T) * 4 * (size_t)Jacobi<T>::cells(dp))) : s.X0;
     return s;
 }
 
@@ -1982,23 +2134,30 @@ struct PsdCheck {
     int* vok;
 };
 
-// FP64 Jacobi of the input block X0 (FP32 eigensolves only), in the place of
-// the FP32 X and V, which are dead: that matrix (returned) leaves with the
-// eigenvalues on its diagonal, V64 with the eigenvectors.
-static __device__ __noinline__ double* psd_redo_fp64(PsdSmem<float>& sm, int dp, int ld)
+// FP64 Jacobi of the input block X0 (FP32 eigensolves only): the cells in the
+// place of the FP32 V and cells, which are dead, the eigenvectors in V64
+// (columns, stride dp), the positive parts of the eigenvalues in lam64.
+static __device__ __noinline__ void psd_redo_fp64(PsdSmem<float>& sm, int dp, double* lam64)
 {
-    double* X64 = reinterpret_cast<double*>(sm.X);
+    double* c0 = reinterpret_cast<double*>(sm.V);
+    const Jacobi<double> J(c0, c0 + 4 * Jacobi<double>::cells(dp), sm.V64, reinterpret_cast<double*>(sm.scratch), dp, dp);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();
-    for (int i = threadIdx.x; i < dp * ld; i += blockDim.x) X64[i] = (double)sm.X0[i];
+    for (int j = warp; j < dp; j += nw)
+        for (int i = lane; i < dp; i += 32) {
+            if (i >= j) J.put(i, j, (double)sm.X0[i * (dp + 1) + j]);
+            J.V[j * dp + i] = i == j ? 1.0 : 0.0;
+        }
+    int cur;
+    jacobi_sweeps<double>(J, sm.red, 1e-26, 20, cur);
+    for (int i = threadIdx.x; i < dp; i += blockDim.x) lam64[i] = fmax(J.dg[cur * dp + J.slot_of(i)], 0.0);
     __syncthreads();
-    jacobi_block<double>(X64, sm.V64, dp, ld, reinterpret_cast<double*>(sm.scratch), sm.red, 1e-26, 20);
-    return X64;
 }
 
-// (V W V^T)(i, j) for i >= j, W = diag(l), from V and U = V W (row stride ld): every entry of
-// the lower triangle by one thread, four rows of a column together; columns with W = 0 skipped.
+// V diag(l) V^T, the entries (i, j), i >= j, of its leading d x d part, from V's columns (stride
+// ldv): four rows of one column a thread; eigenvectors with l = 0 are skipped.
 template <typename T, class Emit>
-__device__ __forceinline__ void psd_rebuild(const T* U, const T* V, const T* l, int d, int dp, int ld, Emit emit)
+__device__ __forceinline__ void psd_rebuild(const T* V, const T* l, int d, int dp, int ldv, Emit emit)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int i0 = 4 * warp; i0 < d; i0 += 4 * nw)
@@ -2006,9 +2165,10 @@ __device__ __forceinline__ void psd_rebuild(const T* U, const T* V, const T* l, 
             T a[4] = {0, 0, 0, 0};
             for (int k = 0; k < dp; ++k) {
                 if (l[k] == T(0)) continue;
-                const T v = V[j * ld + k];
+                const T* c = V + k * ldv;
+                const T v = l[k] * c[j];
 #pragma unroll
-                for (int h = 0; h < 4; ++h) a[h] = fmaT(U[min(i0 + h, d - 1) * ld + k], v, a[h]);
+                for (int h = 0; h < 4; ++h) a[h] = fmaT(c[min(i0 + h, d - 1)], v, a[h]);
             }
 #pragma unroll
             for (int h = 0; h < 4; ++h)
@@ -2076,8 +2236,20 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
             const int o = n + ro(P.s_off + k);
             const int dp = d + (d & 1);
             const int ld = dp + 1;  // odd row stride: column walks are free of bank conflicts
+            const int ldv = psd_ldv<T>(dp);
             PsdSmem<T> sm = psd_layout<T>(psd_base, d > PSD_MAX ? P.psd_big + ro(P.big_off + k) : nullptr, dp);
+            const Jacobi<T> J(sm.cell[0], sm.cell[1], sm.V, sm.scratch, dp, ldv);
             const double isq2 = 0.70710678118654752440;
+            // Warm start: successive projections of a block see nearby matrices, so the
+            // eigenvectors Vp of the last converged decomposition nearly diagonalise this one.
+            // The sweeps run on Vp^T X Vp and accumulate onto V = Vp: the same eigenpairs, found in
+            // a few sweeps instead of a dozen.  vok[k] counts the generations since the last cold
+            // start; V loses orthogonality by a few roundings per generation, so every
+            // PSD_WARM_GEN-th decomposition starts cold again.
+            constexpr int PSD_WARM_GEN = sizeof(T) == 4 ? 16 : 64;
+            T* Vp = ck.vbase ? reinterpret_cast<T*>(ck.vbase + ro(ck.voff + k)) : nullptr;
+            const int gen = Vp ? *(volatile const int*)(ck.vok + k) : 0;
+            const bool warm = gen > 0 && gen < PSD_WARM_GEN;
             __syncthreads();
             for (int j = warp; j < dp; j += nwb)  // column j of the lower triangle: consecutive in svec
                 for (int i = j + lane; i < dp; i += 32) {
@@ -2088,72 +2260,79 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                         const T v = T(2) * wt - w;
                         val = i == j ? v : (T)((double)v * isq2);
                     }
-                    sm.X[i * ld + j] = val;
-                    sm.X[j * ld + i] = val;
-                    if constexpr (sizeof(T) == 4) {
+                    if (warm || sizeof(T) == 4) {
                         sm.X0[i * ld + j] = val;
                         sm.X0[j * ld + i] = val;
                     }
+                    if (!warm) J.put(i, j, val);
                 }
-            __syncthreads();
-            const double tol2 = sizeof(T) == 8 ? 1e-26 : 1e-11;
-            // Warm start: successive projections of a block see nearby matrices, so the
-            // eigenvectors Vp of the last converged decomposition nearly diagonalise this one.
-            // X <- Vp^T X Vp (its lower triangle) and V <- Vp, then the sweeps accumulate onto V:
-            // the same eigenpairs, found in a few sweeps instead of a dozen.  vok[k] counts the
-            // generations since the last cold start; V loses orthogonality by a few roundings
-            // per generation, so every PSD_WARM_GEN-th decomposition starts cold again.
-            constexpr int PSD_WARM_GEN = sizeof(T) == 4 ? 16 : 64;
-            T* Vp = ck.vbase ? reinterpret_cast<T*>(ck.vbase + ro(ck.voff + k)) : nullptr;
-            const int gen = Vp ? *(volatile const int*)(ck.vok + k) : 0;
-            const bool warm = gen > 0 && gen < PSD_WARM_GEN;
             if (warm) {
-                for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // V <- X Vp, four rows a thread
-                    for (int j = lane; j < dp; j += 32) {
+                constexpr int VW = 16 / (int)sizeof(T);
+                struct alignas(16) Vec {
+                    T x[VW];
+                };
+                __syncthreads();
+                for (int j0 = 4 * warp; j0 < dp; j0 += 4 * nwb)  // T <- X Vp, four columns a thread
+                    for (int i = lane; i < dp; i += 32) {
                         T a[4] = {0, 0, 0, 0};
-                        for (int l = 0; l < dp; ++l) {
-                            const T v = Vp[l * ld + j];
+                        for (int l = 0; l < dp; l += VW) {
+                            Vec v[4];
 #pragma unroll
-                            for (int h = 0; h < 4; ++h) a[h] = fmaT(sm.X[min(i0 + h, dp - 1) * ld + l], v, a[h]);
+                            for (int h = 0; h < 4; ++h)
+                                v[h] = *reinterpret_cast<const Vec*>(Vp + min(j0 + h, dp - 1) * ldv + l);
+#pragma unroll
+                            for (int u = 0; u < VW; ++u) {
+                                const T x = l + u < dp ? sm.X0[(l + u) * ld + i] : T(0);
+#pragma unroll
+                                for (int h = 0; h < 4; ++h) a[h] = l + u < dp ? fmaT(x, v[h].x[u], a[h]) : a[h];
+                            }
                         }
 #pragma unroll
                         for (int h = 0; h < 4; ++h)
-                            if (i0 + h < dp) sm.V[(i0 + h) * ld + j] = a[h];
+                            if (j0 + h < dp) sm.V[i * ld + j0 + h] = a[h];
                     }
                 __syncthreads();
-                for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // X <- Vp^T V, lower triangle
+                for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // Vp^T T, lower triangle
                     for (int j = lane; j < min(i0 + 4, dp); j += 32) {
                         T a[4] = {0, 0, 0, 0};
-                        for (int l = 0; l < dp; ++l) {
-                            const T v = sm.V[l * ld + j];
+                        for (int l = 0; l < dp; l += VW) {
+                            Vec v[4];
 #pragma unroll
-                            for (int h = 0; h < 4; ++h) a[h] = fmaT(Vp[l * ld + min(i0 + h, dp - 1)], v, a[h]);
+                            for (int h = 0; h < 4; ++h)
+                                v[h] = *reinterpret_cast<const Vec*>(Vp + min(i0 + h, dp - 1) * ldv + l);
+#pragma unroll
+                            for (int u = 0; u < VW; ++u) {
+                                const T x = l + u < dp ? sm.V[(l + u) * ld + j] : T(0);
+#pragma unroll
+                                for (int h = 0; h < 4; ++h) a[h] = l + u < dp ? fmaT(v[h].x[u], x, a[h]) : a[h];
+                            }
                         }
 #pragma unroll
                         for (int h = 0; h < 4; ++h)
-                            if (i0 + h < dp && j <= i0 + h) sm.X[(i0 + h) * ld + j] = a[h];
+                            if (i0 + h < dp && j <= i0 + h) J.put(i0 + h, j, a[h]);
                     }
                 __syncthreads();
-                for (int i = warp; i < dp; i += nwb)
-                    for (int j = lane; j < dp; j += 32) sm.V[i * ld + j] = Vp[i * ld + j];
-                __syncthreads();
+                for (int i = threadIdx.x; i < dp * ldv; i += blockDim.x) sm.V[i] = Vp[i];
+            } else {
+                for (int j = warp; j < dp; j += nwb)
+                    for (int i = lane; i < ldv; i += 32) sm.V[j * ldv + i] = i == j ? T(1) : T(0);
             }
-            const bool conv = jacobi_block<T>(sm.X, sm.V, dp, ld, sm.scratch, sm.red, tol2,
-                                              d > PSD_MAX ? 30 : (sizeof(T) == 8 ? 20 : 15), warm);
+            int cur;
+            const bool conv = jacobi_sweeps<T>(J, sm.red, sizeof(T) == 8 ? 1e-26 : 1e-11,
+                                               d > PSD_MAX ? 30 : (sizeof(T) == 8 ? 20 : 15), cur);
             if (Vp) {
                 if (conv)
-                    for (int i = warp; i < dp; i += nwb)
-                        for (int j = lane; j < dp; j += 32) Vp[i * ld + j] = sm.V[i * ld + j];
+                    for (int i = threadIdx.x; i < dp * ldv; i += blockDim.x) Vp[i] = sm.V[i];
                 if (threadIdx.x == 0) ck.vok[k] = conv ? (warm ? gen + 1 : 1) : 0;
             }
             for (int i = threadIdx.x; i < dp; i += blockDim.x) {
-                const T l = sm.X[i * ld + i];
+                const T l = J.dg[cur * dp + J.slot_of(i)];
                 sm.lam[i] = l > T(0) ? l : T(0);
             }
             if constexpr (sizeof(T) == 4) {
                 // FP64 recheck of the FP32 eigenpairs: ||X V - V diag(l)||_F / ||X||_F
-                for (int i = warp; i < dp; i += nwb)
-                    for (int j = lane; j < dp; j += 32) sm.V64[i * ld + j] = (double)sm.V[i * ld + j];
+                for (int j = warp; j < dp; j += nwb)
+                    for (int i = lane; i < dp; i += 32) sm.V64[i * ld + j] = (double)sm.V[j * ldv + i];
                 __syncthreads();
                 double r2 = 0.0, x2 = 0.0;
                 // a warp takes two rows of X0: each lane widens its entries once and hands them round,
@@ -2161,7 +2340,7 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                 for (int i0 = 2 * warp; i0 < dp; i0 += 2 * nwb)
                     for (int k0 = 0; k0 < dp; k0 += 32) {
                         const int kk = min(k0 + lane, dp - 1);
-                        const double lk = (double)sm.X[kk * ld + kk];
+                        const double lk = (double)J.dg[cur * dp + J.slot_of(kk)];
                         double a0 = -sm.V64[i0 * ld + kk] * lk, a1 = -sm.V64[(i0 + 1) * ld + kk] * lk;
                         for (int j0 = 0; j0 < dp; j0 += 32) {
                             const int jl = min(j0 + lane, dp - 1), jn = min(32, dp - j0);
@@ -2183,21 +2362,13 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                 if (threadIdx.x == 0 && ck.resid)
                     atomicMax((unsigned long long*)ck.resid, (unsigned long long)__double_as_longlong(rel));
                 if (rel > ck.tol && ck.redo) {
-                    double* X64 = psd_redo_fp64(sm, dp, ld);
+                    double* lam64 = reinterpret_cast<double*>(sm.lam);
+                    psd_redo_fp64(sm, dp, lam64);
                     if (threadIdx.x == 0) {
                         atomicAdd((unsigned long long*)ck.redo, 1ull);
                         if (Vp) ck.vok[k] = 0;  // the FP32 eigenvectors were not good enough to start from
                     }
-                    double* lam64 = reinterpret_cast<double*>(sm.scratch);  // the sweeps are over
-                    for (int i = threadIdx.x; i < dp; i += blockDim.x) {
-                        const double l = X64[i * ld + i];
-                        lam64[i] = l > 0.0 ? l : 0.0;
-                    }
-                    __syncthreads();
-                    for (int i = warp; i < dp; i += nwb)
-                        for (int j = lane; j < dp; j += 32) X64[i * ld + j] = sm.V64[i * ld + j] * lam64[j];
-                    __syncthreads();
-                    psd_rebuild<double>(X64, sm.V64, lam64, d, dp, ld, [&](int i, int j, double x) {
+                    psd_rebuild<double>(sm.V64, lam64, d, dp, dp, [&](int i, int j, double x) {
                         const int e = o + svec_index(d, i, j);
                         T w, wt;
                         op.load(e, w, wt);
@@ -2208,10 +2379,7 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                 }
             }
             __syncthreads();
-            for (int i = warp; i < dp; i += nwb)  // X is dead: V diag(lam) in its place
-                for (int j = lane; j < dp; j += 32) sm.X[i * ld + j] = sm.V[i * ld + j] * sm.lam[j];
-            __syncthreads();
-            psd_rebuild<T>(sm.X, sm.V, sm.lam, d, dp, ld, [&](int i, int j, T x) {
+            psd_rebuild<T>(sm.V, sm.lam, d, dp, ldv, [&](int i, int j, T x) {
                 const int e = o + svec_index(d, i, j);
                 T w, wt;
                 op.load(e, w, wt);

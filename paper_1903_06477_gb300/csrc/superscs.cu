@@ -804,7 +804,8 @@ struct DevInfo {
 template <typename T>
 static size_t dyn_smem(const HostProb& H, int threads, bool tma)
 {
-    const size_t psd = H.s.empty() ? 0 : psd_smem_bytes<T>();
+    size_t psd = 0;
+    for (int d : H.s) psd = std::max(psd, psd_smem_bytes<T>(d));
     const size_t stage = tma ? (size_t)(threads / 32) * 2 * tma_stage_bytes<T>() : 0;
     return std::max(psd, stage);
 }
@@ -1605,10 +1606,11 @@ static int batch_finish_setup(scs_batch* b, const scs_settings* settings, scs_ba
         return b->H[x].nnz + b->H[x].n + b->H[x].m > b->H[y].nnz + b->H[y].n + b->H[y].m;
     });
     b->has32 = settings->precision == SCS_MIXED;
-    bool any_psd = false;
-    for (auto& h : b->H) any_psd |= !h.s.empty();
-    b->dyn64 = any_psd ? psd_smem_bytes<double>() : 0;
-    b->dyn32 = any_psd && b->has32 ? psd_smem_bytes<float>() : 0;
+    for (auto& h : b->H)
+        for (int d : h.s) {
+            b->dyn64 = std::max(b->dyn64, psd_smem_bytes<double>(d));
+            if (b->has32) b->dyn32 = std::max(b->dyn32, psd_smem_bytes<float>(d));
+        }
     if (b->has32) b->dyn64 = std::max(b->dyn64, b->dyn32);
     if ((rc = config_kernels<double>(b->err)) || (b->has32 && (rc = config_kernels<float>(b->err)))) {
         memcpy(g_err, b->err, 512);
