@@ -376,7 +376,7 @@ static void plan_cb(int rows, int cols, const std::vector<int>& rp, const std::v
     for (int attempt = 0; attempt < 8 && cw >= 64; ++attempt) {
         const int ncb = (cols + cw - 1) / cw;
         const int cw2 = ((cols + ncb - 1) / ncb + 3) & ~3;
-        if (!force && nnz < 1024LL * G * ncb) return;
+        if (!force && nnz < 1024LL * G * ncb) break;  // C may hold the attempt before: cleared below
         const long long max_e = build_cb(rows, cols, rp, ci, vx, rb, nw, cw2, S, C);
         if (max_e < 0) break;
         const long long off_x = 4LL * C.ms;
