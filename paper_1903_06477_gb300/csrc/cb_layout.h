@@ -30,7 +30,13 @@ struct CbLayout {
 // column-blocked layout (grid team)
 // ---------------------------------------------------------------------------
 
-// contiguous row ranges for G CTAs, balanced on (entries + 2) per row
+// contiguous row ranges for G CTAs, balanced on (entries + 2) per row.  A range
+// that begins with short rows and ends with long ones, or the other way round
+// (16 times as many entries: the bound rows and the dense rows of a cone
+// program meet there), ends or begins where they meet: a segment has one
+// number of lanes per row, and with a few lanes the long rows of that one CTA
+// took as long as the rest of the product (LASSO design rows of 1000 entries
+// after rows of 2: 12.6 us a product in FP64, 6.1 us so).
 static std::vector<int> cb_row_bounds(int rows, const std::vector<int>& rp, int G)
 {
     std::vector<int> rb(G + 1, 0);
@@ -42,6 +48,32 @@ static std::vector<int> cb_row_bounds(int rows, const std::vector<int>& rp, int 
         rb[b] = r;
     }
     rb[G] = rows;
+    auto len = [&](int i) { return rp[i + 1] - rp[i]; };
+    auto weight = [&](int i) { return (long long)rp[i] + 2LL * i; };
+    for (int b = 0; b < G; ++b) {
+        const int r0 = rb[b], r1 = rb[b + 1], n = r1 - r0;
+        if (n < 2) continue;
+        // extremes of the rows from each end, up to the only place where they can meet
+        int c = -1;
+        const bool up = len(r1 - 1) > len(r0);
+        const int lo = up ? len(r0) : len(r1 - 1), hi = up ? len(r1 - 1) : len(r0);
+        if (hi < 64 || hi < 16 * std::max(lo, 1)) continue;
+        int most = 0, least = hi;  // entries of the short side's and of the long side's rows
+        for (int i = 0; i < n; ++i) {
+            const int row = up ? r0 + i : r1 - 1 - i;
+            if (c < 0 && len(row) > hi / 4) c = i;
+            if (c < 0) most = std::max(most, len(row));
+            else least = std::min(least, len(row));
+        }
+        if (c <= 0 || least < 16 * std::max(most, 1)) continue;
+        const int cut = up ? r0 + c : r1 - c;
+        // the lighter side goes to the neighbour on its own end
+        if ((weight(cut) - weight(r0) < weight(r1) - weight(cut) && b > 0) || b == G - 1) {
+            if (b > 0) rb[b] = cut;
+        } else {
+            rb[b + 1] = cut;
+        }
+    }
     return rb;
 }
 
@@ -73,9 +105,19 @@ struct CbBuckets {
     }
 };
 
+// Fixed cost of a slice with V lanes a row, in half steps: its start and its flush, and one shuffle and
+// addition a level of the sum over its V lanes.
+static int cb_slice_cost(int V)
+{
+    int levels = 0;
+    while ((1 << levels) < V) ++levels;
+    return 3 + 2 * levels;
+}
+
 // Deal slices (work = steps) to nw warps, largest first to the least-loaded
-// warp.  Returns the warp of each slice; loads accumulate 2 * steps + 3.
-static void cb_deal(const std::vector<int>& steps, int nw, std::vector<int>& warp, std::vector<long long>& load)
+// warp.  Returns the warp of each slice; loads accumulate 2 * steps + fixed.
+static void cb_deal(const std::vector<int>& steps, int nw, int fixed, std::vector<int>& warp,
+                    std::vector<long long>& load)
 {
     load.assign(nw, 0);
     warp.resize(steps.size());
@@ -84,7 +126,7 @@ static void cb_deal(const std::vector<int>& steps, int nw, std::vector<int>& war
         for (int w = 1; w < nw; ++w)
             if (load[w] < load[best]) best = w;
         warp[s] = best;
-        load[best] += 2LL * steps[s] + 3;
+        load[best] += 2LL * steps[s] + fixed;
     }
 }
 
@@ -97,41 +139,40 @@ static void cb_slice_steps(const CbBuckets& bk, int k, int R, const std::vector<
     for (int sl = 0; sl < ns; ++sl) steps[sl] = (bk.cnt[(size_t)k * R + rows[(size_t)sl * H]] + V - 1) / V;
 }
 
-// Lanes per row for the column-blocked layout: the V in {1, 2, 4, 8} with the
-// least estimated time on a sample of CTAs -- per segment, the busiest
-// warp's load plus eight times the mean load.  Segments are computed from
-// shared memory while the matrix stream is the bound, so padding (the mean)
-// weighs more than imbalance.
-static int cb_pick_lanes(const std::vector<int>& rp, const std::vector<int>& ci, const std::vector<int>& rb, int nw,
-                         int ncb, int cw)
+// Lanes per row of one segment: the V in {1, 2, 4, 8, 16, 32} with the least
+// estimated time -- the busiest warp's load plus eight times the mean load.
+// Segments are computed from shared memory while the matrix stream is the
+// bound, so padding (the mean) weighs more than imbalance.  The choice belongs
+// to the segment and goes up to a warp a row because a matrix can have both
+// kinds of row: with at most 8 lanes, and one choice for the matrix, the 1000
+// entries of a LASSO design row were 125 steps of one warp while the others
+// waited (A^T of the 2202 x 2001 LASSO in FP64: 9.0 us a product, 5.3 us now).
+static long long cb_lanes_cost(const std::vector<int>& steps, int nw, int fixed, std::vector<int>& warp,
+                               std::vector<long long>& load)
 {
-    const int G = (int)rb.size() - 1;
-    const int stride = std::max(1, G / 16);
-    long long cost[4] = {0, 0, 0, 0};
-    CbBuckets bk;
-    std::vector<int> rows, steps, warp;
-    std::vector<long long> load;
-    for (int b = 0; b < G; b += stride) {
-        const int r0 = rb[b], R = rb[b + 1] - r0;
-        bk.build(r0, R, ncb, cw, rp, ci);
-        for (int k = 0; k < ncb; ++k) {
-            bk.sorted_rows(k, R, rows);
-            for (int vi = 0; vi < 4; ++vi) {
-                cb_slice_steps(bk, k, R, rows, 1 << vi, steps);
-                cb_deal(steps, nw, warp, load);
-                long long mx = 0, sum = 0;
-                for (long long l : load) {
-                    mx = std::max(mx, l);
-                    sum += l;
-                }
-                cost[vi] += mx + 8 * sum / nw;
-            }
+    cb_deal(steps, nw, fixed, warp, load);
+    long long mx = 0, sum = 0;
+    for (long long l : load) {
+        mx = std::max(mx, l);
+        sum += l;
+    }
+    return mx + 8 * sum / nw;
+}
+
+static int cb_pick_lanes(const CbBuckets& bk, int k, int R, const std::vector<int>& rows, int nw,
+                         std::vector<int>& steps, std::vector<int>& warp, std::vector<long long>& load)
+{
+    int best = 1;
+    long long best_cost = -1;
+    for (int V = 1; V <= 32; V *= 2) {
+        cb_slice_steps(bk, k, R, rows, V, steps);
+        const long long cost = cb_lanes_cost(steps, nw, cb_slice_cost(V), warp, load);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = V;
         }
     }
-    int best = 0;
-    for (int vi = 1; vi < 4; ++vi)
-        if (cost[vi] < cost[best]) best = vi;
-    return 1 << best;
+    return best;
 }
 
 // metadata words per segment for ns slices of H rows (layout of Cblk)
@@ -214,17 +255,15 @@ static long long build_cb(int rows, int cols, const std::vector<int>& rp, const 
     (void)rows;
     const int G = (int)rb.size() - 1;
     const int ncb = (cols + cw - 1) / cw;
-    const int V = cb_pick_lanes(rp, ci, rb, nw, ncb, cw);
-    const int H = 32 / V;
     C.ncb = ncb;
     C.cw = cw;
     C.cols = cols;
     C.nw = nw;
-    C.V = V;
     C.S = S;
     C.rbnd = rb;
     struct Seg {
         long long e0, e1;
+        int V;                   // lanes per row
         std::vector<int> words;  // [4] onwards of the segment's metadata
     };
     std::vector<Seg> segs((size_t)G * ncb);
@@ -243,11 +282,14 @@ static long long build_cb(int rows, int cols, const std::vector<int>& rp, const 
     // pass 1: the entries of every segment
     parallel([&](int b) {
         thread_local CbBuckets bk;
-        thread_local std::vector<int> rows_k, steps;
+        thread_local std::vector<int> rows_k, steps, warp;
+        thread_local std::vector<long long> load;
         const int r0 = rb[b], R = rb[b + 1] - r0;
         bk.build(r0, R, ncb, cw, rp, ci);
         for (int k = 0; k < ncb; ++k) {
             bk.sorted_rows(k, R, rows_k);
+            const int V = cb_pick_lanes(bk, k, R, rows_k, nw, steps, warp, load);
+            segs[(size_t)b * ncb + k].V = V;
             cb_slice_steps(bk, k, R, rows_k, V, steps);
             long long e = 0;
             for (int st : steps) e += 32LL * st;
@@ -273,13 +315,14 @@ static long long build_cb(int rows, int cols, const std::vector<int>& rp, const 
         bk.build(r0, R, ncb, cw, rp, ci);
         for (int k = 0; k < ncb; ++k) {
             bk.sorted_rows(k, R, rows_k);
+            Seg& sg = segs[(size_t)b * ncb + k];
+            const int V = sg.V, H = 32 / V;
             cb_slice_steps(bk, k, R, rows_k, V, steps);
-            cb_deal(steps, nw, warp, load);
+            cb_deal(steps, nw, cb_slice_cost(V), warp, load);
             const int ns = (int)steps.size();
             order.resize(ns);
             std::iota(order.begin(), order.end(), 0);
             std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return warp[a] < warp[c]; });
-            Seg& sg = segs[(size_t)b * ncb + k];
             std::vector<int> wstart(nw + 1, 0), sstart(ns + 1, 0);
             std::vector<uint16_t> srow((size_t)ns * H, 0xFFFF);
             int w = 0, t = 0;
@@ -305,7 +348,7 @@ static long long build_cb(int rows, int cols, const std::vector<int>& rp, const 
             sstart[ns] = t;
             while (w <= nw) wstart[w++] = ns;
             sg.words.clear();
-            sg.words.push_back(ns);
+            sg.words.push_back(ns | (H << 16));  // ns <= acc_rows < 65535
             sg.words.insert(sg.words.end(), wstart.begin(), wstart.end());
             sg.words.insert(sg.words.end(), sstart.begin(), sstart.end());
             for (int i = 0; i < ns * H; i += 2) {
@@ -367,7 +410,7 @@ static void plan_cb(int rows, int cols, const std::vector<int>& rp, const std::v
     const size_t acc_bytes = ((size_t)2 * nv * std::max(acc_rows, 1) * esize + 15) & ~size_t(15);
     if (acc_bytes + 4096 > dyn_max) return;
     const long long stage_avail = (long long)((dyn_max - acc_bytes) / S) & ~15LL;
-    // metadata bound: at most ceil(acc_rows / H) slices, H >= 4
+    // metadata, as estimated with ceil(acc_rows / 4) slices (the attempts check the true size)
     const int ms_cap = (cb_meta_words(nw, (acc_rows + 3) / 4, 4) + 16 + 3) & ~3;
     const double per_col = esize + 1.15 * (2 + esize) * (double)nnz_cta / std::max(cols, 1);
     long long budget = stage_avail - 4LL * ms_cap - 64 - 2LL * E * esize;
@@ -398,6 +441,34 @@ static void plan_cb(int rows, int cols, const std::vector<int>& rp, const std::v
     C = CbLayout();
 }
 
+
+// Lanes per row of a tiled matrix, one choice for all its tiles: the V in {1, 2, 4, 8} with the least cost
+// (as for a segment) on a sample of row ranges.
+static int tile_pick_lanes(const std::vector<int>& rp, const std::vector<int>& ci, const std::vector<int>& rb, int nw,
+                           int ncb, int cw)
+{
+    const int G = (int)rb.size() - 1;
+    const int stride = std::max(1, G / 16);
+    long long cost[4] = {0, 0, 0, 0};
+    CbBuckets bk;
+    std::vector<int> rows, steps, warp;
+    std::vector<long long> load;
+    for (int b = 0; b < G; b += stride) {
+        const int r0 = rb[b], R = rb[b + 1] - r0;
+        bk.build(r0, R, ncb, cw, rp, ci);
+        for (int k = 0; k < ncb; ++k) {
+            bk.sorted_rows(k, R, rows);
+            for (int vi = 0; vi < 4; ++vi) {
+                cb_slice_steps(bk, k, R, rows, 1 << vi, steps);
+                cost[vi] += cb_lanes_cost(steps, nw, 3, warp, load);
+            }
+        }
+    }
+    int best = 0;
+    for (int vi = 1; vi < 4; ++vi)
+        if (cost[vi] < cost[best]) best = vi;
+    return 1 << best;
+}
 
 // ---------------------------------------------------------------------------
 // two-dimensional tiles (grid team)
@@ -470,7 +541,7 @@ static bool build_tile(int cols, const std::vector<int>& rp, const std::vector<i
                 }
                 if (ns == 0) return false;
                 sub.assign(steps.begin() + sl, steps.begin() + sl + ns);
-                cb_deal(sub, nw, warp, load);
+                cb_deal(sub, nw, 3, warp, load);
                 order.resize(ns);
                 std::iota(order.begin(), order.end(), 0);
                 std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return warp[a] < warp[c]; });
@@ -591,7 +662,7 @@ static void plan_tile(int rows, int cols, const std::vector<int>& rp, const std:
         Split sp;
         split(cd.second, sp);
         const int Cn = sp.Cn, R = G / Cn;
-        const int V = cb_pick_lanes(rp, ci, sp.rb, nw, Cn, sp.cw);
+        const int V = tile_pick_lanes(rp, ci, sp.rb, nw, Cn, sp.cw);
         const int H = 32 / V;
         // metadata share of a stage from the mean slice (sampled row blocks):
         // 1 + H/2 words per slice against 32 x steps entries of 2 + esize bytes

@@ -87,7 +87,7 @@ struct DevState {
 // owns the contiguous rows [rbnd[b], rbnd[b+1]); the columns are cut into ncb
 // blocks of cw.  A "segment" is one (CTA, column block) pair: the CTA's rows
 // that have entries in the block, sorted by their count there (descending),
-// packed as slices of H = 32 / V rows with element j of slice row r at
+// packed as slices of H = 32 / V rows (V chosen for each segment) with element j of slice row r at
 // step (slice start + j / V), lane (j % V) * H + r, 32 entries per step, and
 // its column stored as a 16-bit offset inside the block (padding: value 0,
 // offset 0).  The slices of a segment are dealt to the CTA's warps (largest
@@ -96,7 +96,7 @@ struct DevState {
 //
 // Each segment has ms 32-bit words of metadata at meta + g * ms:
 //   [0] E0   [1] E1   [2], [3] E0, E1 of the CTA's segment (k + S) mod ncb
-//   [4] ns: slices    [5 .. 5+nw] first slice of each warp (nw+1 values)
+//   [4] ns slices + (H << 16)   [5 .. 5+nw] first slice of each warp (nw+1 values)
 //   [6+nw .. 6+nw+ns] slice start steps from E0 (ns+1 values)
 //   then ns * H 16-bit row indices inside the CTA's range (0xFFFF: none),
 //   two per word, low half first.
@@ -121,7 +121,7 @@ struct Cblk {
     int cw;           // columns per block (multiple of 4)
     int cols;         // columns of the matrix
     int nw;           // compute warps per CTA (the CTA has nw + 1 warps)
-    int V;            // lanes per row
+    int V;            // lanes per row (tiles; the segments name their own)
     int acc_rows;     // partial-sum entries per buffer (largest row range); 2 buffers per vector
     int ms;           // metadata words per segment (multiple of 4)
     int S;            // stages in the copy ring (2..CB_MAX_STAGES)
@@ -216,7 +216,7 @@ struct DevWork {
     double *x_out, *y_out, *s_out, *u_out; // results (FP64)
     unsigned char* psd_v;  // PSD blocks: eigenvectors of the last converged decomposition (warm starts)
     int* psd_vok;          // per PSD block: 0 if psd_v holds nothing, else warm-start generations
-    double* partials;      // [2][KMAX][blocks] block partials, then [2][KMAX] results
+    double* partials;      // [2][KMAX][blocks] block partials
     unsigned* bar;
     int* abort_flag;
     DevState* st;
@@ -433,7 +433,7 @@ __device__ __forceinline__ void sell_tma(const Team& tm, const Sell<T>& S, XF& x
 // shared array itself so the loads are 32-bit-addressed shared loads and the
 // hot loop touches no local memory.
 template <typename T>
-__device__ __forceinline__ void cb_segment(int nw, int H, unsigned mt_off, unsigned xs_off, unsigned col_off,
+__device__ __forceinline__ void cb_segment(int nw, unsigned mt_off, unsigned xs_off, unsigned col_off,
                                            unsigned val_off, unsigned acc_off)
 {
     extern __shared__ __align__(128) unsigned char cb_sm[];
@@ -443,7 +443,7 @@ __device__ __forceinline__ void cb_segment(int nw, int H, unsigned mt_off, unsig
     const T* sval = (const T*)(cb_sm + val_off);
     T* acc = (T*)(cb_sm + acc_off);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int ns = mt[4];
+    const int ns = mt[4] & 0xFFFF, H = mt[4] >> 16;
     const int* wl = mt + 5;
     const int* st = wl + nw + 1;
     const unsigned short* sr = (const unsigned short*)(st + ns + 1);
@@ -502,10 +502,9 @@ __device__ __forceinline__ void cb_segment(int nw, int H, unsigned mt_off, unsig
     for (int s = s0; s < s_hi; ++s) {
         const int t1 = st[s + 1];
         int t = st[s];
-        T a0 = 0, a1 = 0;
         if constexpr (sizeof(T) == 4) {
             // FP32: four steps per trip, the tail predicated (offset 0, value 0)
-            T a2 = 0, a3 = 0;
+            T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
             for (; t < t1; t += 4) {
                 const bool o1 = t + 1 < t1, o2 = t + 2 < t1, o3 = t + 3 < t1;
                 const int c0 = scol[t * 32 + lane];
@@ -521,9 +520,15 @@ __device__ __forceinline__ void cb_segment(int nw, int H, unsigned mt_off, unsig
                 a2 = fmaT(v2, xs[c2], a2);
                 a3 = fmaT(v3, xs[c3], a3);
             }
-            a0 += a2;
-            a1 += a3;
+            T a = (a0 + a2) + (a1 + a3);
+            for (int o = H; o < 32; o <<= 1) a += __shfl_xor_sync(FULL_MASK, a, o);
+            if (lane < H) {
+                const int r = sr[s * H + lane];
+                if (r != 0xFFFF) acc[r] += a;
+            }
         } else {
+            // FP64: two chains
+            T a0 = 0, a1 = 0;
             for (; t + 2 <= t1; t += 2) {
                 const int c0 = scol[t * 32 + lane], c1 = scol[t * 32 + 32 + lane];
                 const T v0 = sval[t * 32 + lane], v1 = sval[t * 32 + 32 + lane];
@@ -531,12 +536,12 @@ __device__ __forceinline__ void cb_segment(int nw, int H, unsigned mt_off, unsig
                 a1 = fmaT(v1, xs[c1], a1);
             }
             if (t < t1) a0 = fmaT(sval[t * 32 + lane], xs[scol[t * 32 + lane]], a0);
-        }
-        T a = a0 + a1;
-        for (int o = H; o < 32; o <<= 1) a += __shfl_xor_sync(FULL_MASK, a, o);
-        if (lane < H) {
-            const int r = sr[s * H + lane];
-            if (r != 0xFFFF) acc[r] += a;
+            T a = a0 + a1;
+            for (int o = H; o < 32; o <<= 1) a += __shfl_xor_sync(FULL_MASK, a, o);
+            if (lane < H) {
+                const int r = sr[s * H + lane];
+                if (r != 0xFFFF) acc[r] += a;
+            }
         }
     }
 }
@@ -554,7 +559,7 @@ template <typename T>
 __device__ bool cb_pass(const GridTeam& tm, const Cblk<T>& C, const T* x, T* acc, unsigned long long pol)
 {
     constexpr int E = 16 / (int)sizeof(T);
-    const int S = C.S, ncb = C.ncb, nw = C.nw, H = 32 / C.V, ms = C.ms, cw = C.cw, cols = C.cols;
+    const int S = C.S, ncb = C.ncb, nw = C.nw, ms = C.ms, cw = C.cw, cols = C.cols;
     const int off_x = C.off_x, off_col = C.off_col, off_val = C.off_val, ar = C.acc_rows;
     const int* meta = C.meta;
     const unsigned short* gcol = C.col;
@@ -648,7 +653,7 @@ __device__ bool cb_pass(const GridTeam& tm, const Cblk<T>& C, const T* x, T* acc
                 }
             }
             const unsigned so = (unsigned)(stage(s) - tm_dsm);
-            cb_segment<T>(nw, H, so, so + off_x + mis * (unsigned)sizeof(T), so + off_col, so + off_val,
+            cb_segment<T>(nw, so, so + off_x + mis * (unsigned)sizeof(T), so + off_col, so + off_val,
                           acc_off + (unsigned)((j & 1) * ar * (int)sizeof(T)));
             __syncwarp();
             if (lane == 0) mbar_arrive(empty(s));

@@ -174,7 +174,8 @@ extern "C" int scs_cb_layout_check(int32_t rows, int32_t cols, const int64_t* Ap
     if (C.ncb == 0) return SCS_OK;  // the layout does not fit: the solver would use sliced ELL
     long long bad = 0;
     auto req = [&](bool c) { if (!c) ++bad; };
-    const int E = 16 / elem_bytes, H = 32 / C.V, S = C.S, nw = compute_warps;
+    const int E = 16 / elem_bytes, S = C.S, nw = compute_warps;
+    int vmax = 1;
     req(C.cw % 4 == 0 && C.cw <= 65536 && (long long)C.ncb * C.cw >= cols && (long long)(C.ncb - 1) * C.cw < cols);
     req(C.dyn() <= (size_t)smem_bytes);
     req((size_t)C.stage_off >= (size_t)2 * vectors * C.acc_rows * elem_bytes && C.stage_off % 16 == 0);
@@ -196,7 +197,10 @@ extern "C" int scs_cb_layout_check(int32_t rows, int32_t cols, const int64_t* Ap
         for (int k = 0; k < C.ncb; ++k) {
             const int len = std::min(C.cw, cols - k * C.cw);
             const int* mt = C.meta.data() + ((size_t)b * C.ncb + k) * C.ms;
-            const int e0 = mt[0], e1 = mt[1], ns = mt[4];
+            const int e0 = mt[0], e1 = mt[1], ns = mt[4] & 0xFFFF, H = mt[4] >> 16;
+            req(H >= 1 && H <= 32 && (H & (H - 1)) == 0);
+            const int V = 32 / std::min(32, std::max(1, H));
+            vmax = std::max(vmax, V);
             req(e0 == prev_end && e1 >= e0 && e0 % 32 == 0 && e1 % 32 == 0);
             req((long long)(e1 - e0) * 2 <= C.off_val - C.off_col &&
                 (long long)(e1 - e0) * elem_bytes <= C.stage_bytes - C.off_val);
@@ -223,7 +227,7 @@ extern "C" int scs_cb_layout_check(int32_t rows, int32_t cols, const int64_t* Ap
                         }
                     for (int r = 0; r < H; ++r) {
                         double sum = 0;
-                        for (int q = 0; q < C.V; ++q) sum += a[q * H + r];
+                        for (int q = 0; q < V; ++q) sum += a[q * H + r];
                         const int rw = sr[sl * H + r];
                         if (rw == 0xFFFF) {
                             req(sum == 0.0);
@@ -244,7 +248,7 @@ extern "C" int scs_cb_layout_check(int32_t rows, int32_t cols, const int64_t* Ap
     stats[0] = bad;
     stats[1] = C.ncb;
     stats[2] = C.cw;
-    stats[3] = C.V;
+    stats[3] = vmax;
     stats[4] = (int64_t)C.col.size();
     stats[5] = (int64_t)C.dyn();
     stats[6] = C.S;
@@ -641,7 +645,7 @@ static void lay_out(Arena& A, const HostProb& H, int mem, bool qr, bool direct, 
     W.y_out = A.take<double>(m);
     W.s_out = A.take<double>(m);
     W.u_out = A.take<double>(nm + 1);
-    W.partials = A.take<double>((size_t)2 * KMAX * std::max(max_blocks, 1) + 2 * KMAX);
+    W.partials = A.take<double>((size_t)2 * KMAX * std::max(max_blocks, 1));
     W.bar = A.take<unsigned>(4);
     W.abort_flag = A.take<int>(4);
     W.st = st_ext ? st_ext : A.take<DevState>(1);
