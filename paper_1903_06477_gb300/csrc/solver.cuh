@@ -184,6 +184,7 @@ struct DevProb {
     unsigned char* psd_big;
     const long long* big_off;
     const long long* v_off;  // byte offset of each PSD block's warm-start eigenvectors in DevWork::psd_v
+    int psd_order;           // the largest PSD order
 };
 
 // Iterative refinement of the FP64 linear solves (SCS_MIXED, FP64 phase): the
@@ -1458,20 +1459,26 @@ __device__ __forceinline__ int svec_index(int d, int i, int j)  // i >= j
     return j * d - j * (j - 1) / 2 + (i - j);
 }
 
-// the sum of x over the CTA, in every thread; red: 33 doubles of shared memory.  The warps' sums are
+// The warps of a CTA that share one PSD block: consecutive threads with a named barrier of their own.
+struct PsdTeam {
+    int tid, nt, bar;
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nt) : "memory"); }
+};
+
+// the sum of x over the team, in every thread; red: 33 doubles of shared memory.  The warps' sums are
 // added by one warp: every thread adding them itself kept the FP64 pipe busy for 4000 cycles.
-__device__ __forceinline__ double block_sum(double x, double* red)
+__device__ __forceinline__ double block_sum(double x, double* red, const PsdTeam& g)
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = g.tid & 31, wid = g.tid >> 5, nw = g.nt >> 5;
     x = warp_sum(x);
-    __syncthreads();
+    g.sync();
     if (lane == 0) red[wid] = x;
-    __syncthreads();
+    g.sync();
     if (wid == 0) {
         const double s = warp_sum(lane < nw ? red[lane] : 0.0);
         if (lane == 0) red[32] = s;
     }
-    __syncthreads();
+    g.sync();
     return red[32];
 }
 
@@ -1571,13 +1578,17 @@ __device__ __forceinline__ float jacobi_tan(float diff, float apq)
 // max_sweeps (FP32: V is updated only, so it must hold the start basis; the
 // matrix has been put).  Returns whether it is (the same value in every
 // thread); dg[slot_of(i)] of buffer `cur` then is eigenvalue i.
+//
+// A function of its own: inlined at its five places it made the solver's kernels so large that their
+// other loops ran slower (sparse program of 1e7 nonzeros in FP64, ten iterations: 28.3 ms, 27.4 ms so).
 template <typename T>
-__device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int max_sweeps, int& cur)
+__device__ __noinline__ bool jacobi_sweeps(const Jacobi<T> J, double* red, double tol2, int max_sweeps, int& cur,
+                                           const PsdTeam g)
 {
     constexpr bool kFast = sizeof(T) == 8;
     constexpr int VW = 16 / (int)sizeof(T);  // rows of V a thread moves at a time
     constexpr int NC = 3;                    // cells of a thread, besides the owned one, whose addresses are kept
-    const int tid = threadIdx.x, nt = blockDim.x, nw = nt >> 5;
+    const int tid = g.tid, nt = g.nt, nw = nt >> 5;
     const int dp = J.dp, half = J.half, ncell = J.ncell;
     struct Cell {
         int k, l, src, dst[4];
@@ -1699,10 +1710,10 @@ __device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int 
         for (int i = tid; i < half; i += nt) s += (double)J.e[i] * (double)J.e[i];
         return 2.0 * s;
     };
-    __syncthreads();
+    g.sync();
     double total = square_sum(0);
     for (int i = tid; i < dp; i += nt) total += (double)J.dg[i] * (double)J.dg[i];
-    total = block_sum(total, red);
+    total = block_sum(total, red, g);
     const int quad = kFast && total > 0.0 && isfinite(total) ? ilogb(total) / 4 : 0;
     if constexpr (kFast) {
         for (int i = tid; i < dp; i += nt) {
@@ -1710,7 +1721,7 @@ __device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int 
             J.sc[i] = scalbn(1.0, -quad);
         }
         total = scalbn(total, -4 * quad);
-        __syncthreads();
+        g.sync();
     }
     // V: a thread has VW rows and every ng-th pair, or all pairs of several row groups
     const int groups = J.ldv / VW;
@@ -1737,9 +1748,9 @@ __device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int 
                     const T f = sc[J.slot_of(j)];
                     for (int i = tid & 31; i < dp; i += 32) J.V[j * J.ldv + i] *= f;
                 }
-            __syncthreads();
+            g.sync();
         }
-        const double off = block_sum(square_sum(cur), red);
+        const double off = block_sum(square_sum(cur), red, g);
         conv = off <= tol2 * total || off == 0.0;
         if (conv || sweep == max_sweeps) break;
         for (int k = tid; k < half; k += nt) {
@@ -1749,7 +1760,7 @@ __device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int 
             }
             rotate(k, J.e[k], ahead(cur, 2 * k, 2 * k + 1), cur);
         }
-        __syncthreads();
+        g.sync();
         for (int rnd = 0; rnd < dp - 1; ++rnd) {
             const T* rot = J.rot + cur * dp;
             const T* src = cur ? buf1 : buf0;
@@ -1850,12 +1861,12 @@ __device__ bool jacobi_sweeps(const Jacobi<T>& J, double* red, double tol2, int 
                         J.isc[cur * dp + b] = J.isc[(cur ^ 1) * dp + a];
                     }
                 }
-            __syncthreads();
+            g.sync();
         }
     }
     if constexpr (kFast) {
         for (int i = tid; i < dp; i += nt) J.dg[cur * dp + i] = scalbn(J.dg[cur * dp + i], 2 * quad);
-        __syncthreads();
+        g.sync();
     }
     return conv;
 }
@@ -2104,6 +2115,37 @@ __host__ __device__ constexpr size_t psd_v_bytes(int d)
     return psd_round(sizeof(T) * (size_t)dp * psd_ldv<T>(dp));
 }
 
+// How a CTA of `threads` threads shares out its PSD blocks, ns of at most order d over `ctas` CTAs, in at
+// most `limit` bytes of shared memory: several blocks at a time, each by a group of its threads, where a
+// CTA has several.  A round of the Jacobi sweeps is a chain of latencies and a block's matrix is small, so
+// a group of 256 threads is hardly slower than 512 (order 64 in FP32, 512 blocks, one group a CTA: 4.0
+// and 3.65 ms; in FP64, where more warps only crowd the pipe, 13.7 and 17.3 ms) and 128 do for small
+// orders (20: 1.01 and 1.10 ms).  A CTA with one block gives it 256 threads, FP32 above order 48 all.
+struct PsdPlan {
+    int threads, groups;
+    unsigned bytes;  // of one group
+};
+template <typename T>
+__host__ __device__ inline PsdPlan psd_plan(int d, int ns, int ctas, int threads, unsigned limit)
+{
+    PsdPlan p{threads, 1, (unsigned)psd_smem_bytes<T>(d)};
+    if (d > PSD_MAX || ns == 0) return p;
+    const int per = (ns + ctas - 1) / ctas;
+    int t = d <= 24 ? 128 : 256;
+    if (per == 1 && (d <= 24 || sizeof(T) == 4)) t = sizeof(T) == 4 && d > 48 ? threads : 256;
+    if (t >= threads || threads % t) return p;
+    p.threads = t;
+    const int room = (int)(limit / p.bytes), most = threads / t < per ? threads / t : per;
+    p.groups = room < most ? (room > 1 ? room : 1) : most;
+    return p;
+}
+__device__ __forceinline__ unsigned dyn_smem_size()
+{
+    unsigned n;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(n));
+    return n;
+}
+
 // smem: the CTA's shared region; big: the block's global workspace, or null
 template <typename T>
 __device__ PsdSmem<T> psd_layout(unsigned char* smem, unsigned char* big, int dp)
@@ -2142,29 +2184,29 @@ struct PsdCheck {
 // FP64 Jacobi of the input block X0 (FP32 eigensolves only): the cells in the
 // place of the FP32 V and cells, which are dead, the eigenvectors in V64
 // (columns, stride dp), the positive parts of the eigenvalues in lam64.
-static __device__ __noinline__ void psd_redo_fp64(PsdSmem<float>& sm, int dp, double* lam64)
+static __device__ __noinline__ void psd_redo_fp64(PsdSmem<float>& sm, int dp, double* lam64, const PsdTeam& g)
 {
     double* c0 = reinterpret_cast<double*>(sm.V);
     const Jacobi<double> J(c0, c0 + 4 * Jacobi<double>::cells(dp), sm.V64, reinterpret_cast<double*>(sm.scratch), dp, dp);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
+    const int lane = g.tid & 31, warp = g.tid >> 5, nw = g.nt >> 5;
+    g.sync();
     for (int j = warp; j < dp; j += nw)
         for (int i = lane; i < dp; i += 32) {
             if (i >= j) J.put(i, j, (double)sm.X0[i * (dp + 1) + j]);
             J.V[j * dp + i] = i == j ? 1.0 : 0.0;
         }
     int cur;
-    jacobi_sweeps<double>(J, sm.red, 1e-26, 20, cur);
-    for (int i = threadIdx.x; i < dp; i += blockDim.x) lam64[i] = fmax(J.dg[cur * dp + J.slot_of(i)], 0.0);
-    __syncthreads();
+    jacobi_sweeps<double>(J, sm.red, 1e-26, 20, cur, g);
+    for (int i = g.tid; i < dp; i += g.nt) lam64[i] = fmax(J.dg[cur * dp + J.slot_of(i)], 0.0);
+    g.sync();
 }
 
 // V diag(l) V^T, the entries (i, j), i >= j, of its leading d x d part, from V's columns (stride
 // ldv): four rows of one column a thread; eigenvectors with l = 0 are skipped.
 template <typename T, class Emit>
-__device__ __forceinline__ void psd_rebuild(const T* V, const T* l, int d, int dp, int ldv, Emit emit)
+__device__ __forceinline__ void psd_rebuild(const T* V, const T* l, int d, int dp, int ldv, const PsdTeam& g, Emit emit)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = g.tid & 31, warp = g.tid >> 5, nw = g.nt >> 5;
     for (int i0 = 4 * warp; i0 < d; i0 += 4 * nw)
         for (int j = lane; j < min(i0 + 4, d); j += 32) {
             T a[4] = {0, 0, 0, 0};
@@ -2232,17 +2274,23 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
         if (lane == 0) op.store(o + dim - 1, wT, wtT, mode == 0 ? tv : (mode == 1 ? T(0) : (T)tb));
         __syncwarp();
     }
-    // PSD blocks: one CTA per block, Jacobi eigen-decomposition in shared memory
-    // (orders above PSD_MAX: in the block's workspace in global memory)
+    // PSD blocks: one group of a CTA's threads per block (psd_groups), Jacobi
+    // eigen-decomposition in shared memory (orders above PSD_MAX: in the block's
+    // workspace in global memory)
     if (P.ns > 0) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwb = blockDim.x >> 5;
-        for (int k = tm.block(); k < P.ns; k += tm.nblocks()) {
+        __syncthreads();  // shared memory is free (earlier users done)
+        const PsdPlan plan = psd_plan<T>(P.psd_order, P.ns, tm.nblocks(), blockDim.x, dyn_smem_size());
+        const int gid = threadIdx.x / plan.threads;
+        const PsdTeam g{(int)threadIdx.x - gid * plan.threads, plan.threads, 1 + gid};
+        const int lane = g.tid & 31, warp = g.tid >> 5, nwb = g.nt >> 5;
+        const int k0 = gid < plan.groups ? tm.block() + gid * tm.nblocks() : P.ns;
+        for (int k = k0; k < P.ns; k += plan.groups * tm.nblocks()) {
             const int d = ro(P.s_dim + k);
             const int o = n + ro(P.s_off + k);
             const int dp = d + (d & 1);
             const int ld = dp + 1;  // odd row stride: column walks are free of bank conflicts
             const int ldv = psd_ldv<T>(dp);
-            PsdSmem<T> sm = psd_layout<T>(psd_base, d > PSD_MAX ? P.psd_big + ro(P.big_off + k) : nullptr, dp);
+            PsdSmem<T> sm = psd_layout<T>(psd_base + gid * plan.bytes, d > PSD_MAX ? P.psd_big + ro(P.big_off + k) : nullptr, dp);
             const Jacobi<T> J(sm.cell[0], sm.cell[1], sm.V, sm.scratch, dp, ldv);
             const double isq2 = 0.70710678118654752440;
             // Warm start: successive projections of a block see nearby matrices, so the
@@ -2255,7 +2303,7 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
             T* Vp = ck.vbase ? reinterpret_cast<T*>(ck.vbase + ro(ck.voff + k)) : nullptr;
             const int gen = Vp ? *(volatile const int*)(ck.vok + k) : 0;
             const bool warm = gen > 0 && gen < PSD_WARM_GEN;
-            __syncthreads();
+            g.sync();
             for (int j = warp; j < dp; j += nwb)  // column j of the lower triangle: consecutive in svec
                 for (int i = j + lane; i < dp; i += 32) {
                     T val = 0;
@@ -2276,7 +2324,7 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                 struct alignas(16) Vec {
                     T x[VW];
                 };
-                __syncthreads();
+                g.sync();
                 for (int j0 = 4 * warp; j0 < dp; j0 += 4 * nwb)  // T <- X Vp, four columns a thread
                     for (int i = lane; i < dp; i += 32) {
                         T a[4] = {0, 0, 0, 0};
@@ -2296,7 +2344,7 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                         for (int h = 0; h < 4; ++h)
                             if (j0 + h < dp) sm.V[i * ld + j0 + h] = a[h];
                     }
-                __syncthreads();
+                g.sync();
                 for (int i0 = 4 * warp; i0 < dp; i0 += 4 * nwb)  // Vp^T T, lower triangle
                     for (int j = lane; j < min(i0 + 4, dp); j += 32) {
                         T a[4] = {0, 0, 0, 0};
@@ -2316,81 +2364,101 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
                         for (int h = 0; h < 4; ++h)
                             if (i0 + h < dp && j <= i0 + h) J.put(i0 + h, j, a[h]);
                     }
-                __syncthreads();
-                for (int i = threadIdx.x; i < dp * ldv; i += blockDim.x) sm.V[i] = Vp[i];
+                g.sync();
+                for (int i = g.tid; i < dp * ldv; i += g.nt) sm.V[i] = Vp[i];
             } else {
                 for (int j = warp; j < dp; j += nwb)
                     for (int i = lane; i < ldv; i += 32) sm.V[j * ldv + i] = i == j ? T(1) : T(0);
             }
             int cur;
             const bool conv = jacobi_sweeps<T>(J, sm.red, sizeof(T) == 8 ? 1e-26 : 1e-11,
-                                               d > PSD_MAX ? 30 : (sizeof(T) == 8 ? 20 : 15), cur);
+                                               d > PSD_MAX ? 30 : (sizeof(T) == 8 ? 20 : 15), cur, g);
             if (Vp) {
                 if (conv)
-                    for (int i = threadIdx.x; i < dp * ldv; i += blockDim.x) Vp[i] = sm.V[i];
-                if (threadIdx.x == 0) ck.vok[k] = conv ? (warm ? gen + 1 : 1) : 0;
+                    for (int i = g.tid; i < dp * ldv; i += g.nt) Vp[i] = sm.V[i];
+                if (g.tid == 0) ck.vok[k] = conv ? (warm ? gen + 1 : 1) : 0;
             }
-            for (int i = threadIdx.x; i < dp; i += blockDim.x) {
+            for (int i = g.tid; i < dp; i += g.nt) {
                 const T l = J.dg[cur * dp + J.slot_of(i)];
                 sm.lam[i] = l > T(0) ? l : T(0);
             }
             if constexpr (sizeof(T) == 4) {
-                // FP64 recheck of the FP32 eigenpairs: ||X V - V diag(l)||_F / ||X||_F
+                // Recheck of the FP32 eigenpairs: ||X V - V diag(l)||_F / ||X||_F.  X, V and l are FP32,
+                // so a product is two FP32 words exactly, and the sums are kept in three words by
+                // error-free additions (Knuth's two-sum), more than FP64's bits; FP64 from there on.
+                // The d^3 multiply-adds in FP64 took as long as the sweeps did (FP64 pipe: 131k cycles
+                // of the SM for order 64; 512 such blocks, one projection: 4.6 ms, 3.8 ms
+                // so).  X is scaled by a power of two so that no word overflows or loses bits to underflow.
+                float* VR = reinterpret_cast<float*>(sm.V64);  // V by rows (stride ld)
                 for (int j = warp; j < dp; j += nwb)
-                    for (int i = lane; i < dp; i += 32) sm.V64[i * ld + j] = (double)sm.V[j * ldv + i];
-                __syncthreads();
-                double r2 = 0.0, x2 = 0.0;
-                // a warp takes two rows of X0: each lane widens its entries once and hands them round,
-                // so the FP64 pipe does the d^3 multiply-adds and d^2 conversions only
-                for (int i0 = 2 * warp; i0 < dp; i0 += 2 * nwb)
-                    for (int k0 = 0; k0 < dp; k0 += 32) {
-                        const int kk = min(k0 + lane, dp - 1);
-                        const double lk = (double)J.dg[cur * dp + J.slot_of(kk)];
-                        double a0 = -sm.V64[i0 * ld + kk] * lk, a1 = -sm.V64[(i0 + 1) * ld + kk] * lk;
-                        for (int j0 = 0; j0 < dp; j0 += 32) {
-                            const int jl = min(j0 + lane, dp - 1), jn = min(32, dp - j0);
-                            const double x0 = (double)sm.X0[i0 * ld + jl], x1 = (double)sm.X0[(i0 + 1) * ld + jl];
-                            if (k0 == 0 && lane < jn) x2 += x0 * x0 + x1 * x1;
-                            for (int j = 0; j < jn; ++j) {
-                                const double v = sm.V64[(j0 + j) * ld + kk];
-                                a0 += __shfl_sync(FULL_MASK, x0, j) * v;
-                                a1 += __shfl_sync(FULL_MASK, x1, j) * v;
-                            }
-                        }
-                        if (k0 + lane < dp) r2 += a0 * a0 + a1 * a1;
+                    for (int i = lane; i < dp; i += 32) VR[i * ld + j] = sm.V[j * ldv + i];
+                double x2 = 0.0, r2 = 0.0;
+                for (int i = warp; i < dp; i += nwb)
+                    for (int j = lane; j < dp; j += 32) x2 += (double)sm.X0[i * ld + j] * (double)sm.X0[i * ld + j];
+                x2 = block_sum(x2, sm.red, g);
+                const int e2 = x2 > 0.0 && isfinite(x2) ? ilogb(x2) / 2 : 0;
+                const float sc1 = scalbnf(1.0f, -(e2 / 2)), sc2 = scalbnf(1.0f, -(e2 - e2 / 2));  // (each in range)
+                const int nk = (dp + 31) >> 5;
+                for (int it = warp; it < nk * ((dp + 3) >> 2); it += nwb) {
+                    // 4 rows by 32 columns a warp, a column a lane
+                    const int i0 = 4 * (it / nk), k = 32 * (it % nk) + lane, kk = min(k, dp - 1);
+                    const float lk = J.dg[cur * dp + J.slot_of(kk)] * sc1 * sc2;
+                    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f}, lo2[4] = {0.f, 0.f, 0.f, 0.f};
+                    auto two_sum = [](float& a, float b) {  // a + b = (a, returned error)
+                        const float t = a + b, z = t - a, e = (a - (t - z)) + (b - z);
+                        a = t;
+                        return e;
+                    };
+                    auto add = [&](int h, float x, float v) {  // (hi, lo, lo2) += x v
+                        const float p = x * v, pe = fmaf(x, v, -p);
+                        const float e = two_sum(hi[h], p);
+                        lo2[h] += two_sum(lo[h], e) + two_sum(lo[h], pe);
+                    };
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) add(h, -lk, VR[min(i0 + h, dp - 1) * ld + kk]);
+                    for (int j = 0; j < dp; ++j) {
+                        const float v = VR[j * ld + kk];
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) add(h, sm.X0[j * ld + min(i0 + h, dp - 1)] * sc1 * sc2, v);
                     }
-                r2 = block_sum(r2, sm.red);
-                x2 = block_sum(x2, sm.red);
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        if (k < dp && i0 + h < dp) {
+                            const double a = (double)hi[h] + ((double)lo[h] + (double)lo2[h]);
+                            r2 += a * a;
+                        }
+                }
+                r2 = scalbn(block_sum(r2, sm.red, g), 2 * e2);
                 // block_sum hands every thread the same sums, so the decision
-                // to decompose the block again in FP64 is uniform in the CTA
+                // to decompose the block again in FP64 is uniform in the group
                 const double rel = x2 > 0.0 ? sqrt(r2 / x2) : 0.0;
-                if (threadIdx.x == 0 && ck.resid)
+                if (g.tid == 0 && ck.resid)
                     atomicMax((unsigned long long*)ck.resid, (unsigned long long)__double_as_longlong(rel));
                 if (rel > ck.tol && ck.redo) {
                     double* lam64 = reinterpret_cast<double*>(sm.lam);
-                    psd_redo_fp64(sm, dp, lam64);
-                    if (threadIdx.x == 0) {
+                    psd_redo_fp64(sm, dp, lam64, g);
+                    if (g.tid == 0) {
                         atomicAdd((unsigned long long*)ck.redo, 1ull);
                         if (Vp) ck.vok[k] = 0;  // the FP32 eigenvectors were not good enough to start from
                     }
-                    psd_rebuild<double>(sm.V64, lam64, d, dp, dp, [&](int i, int j, double x) {
+                    psd_rebuild<double>(sm.V64, lam64, d, dp, dp, g, [&](int i, int j, double x) {
                         const int e = o + svec_index(d, i, j);
                         T w, wt;
                         op.load(e, w, wt);
                         op.store(e, w, wt, (T)(i == j ? x : x * 1.41421356237309504880));
                     });
-                    __syncthreads();
+                    g.sync();
                     continue;
                 }
             }
-            __syncthreads();
-            psd_rebuild<T>(sm.V, sm.lam, d, dp, ldv, [&](int i, int j, T x) {
+            g.sync();
+            psd_rebuild<T>(sm.V, sm.lam, d, dp, ldv, g, [&](int i, int j, T x) {
                 const int e = o + svec_index(d, i, j);
                 T w, wt;
                 op.load(e, w, wt);
                 op.store(e, w, wt, i == j ? x : (T)((double)x * 1.41421356237309504880));
             });
-            __syncthreads();
+            g.sync();
         }
     }
     // exponential cones, one per thread: the psi part lies in K*, so a primal

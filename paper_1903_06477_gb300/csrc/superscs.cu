@@ -596,6 +596,7 @@ static void lay_out(Arena& A, const HostProb& H, int mem, bool qr, bool direct, 
     P.c = A.take<T>(n);
     P.nb = H.nb;
     P.nc = H.nc;
+    P.psd_order = H.s.empty() ? 0 : *std::max_element(H.s.begin(), H.s.end());
     P.f = H.f;
     P.l = H.l;
     P.nq = (int)H.q.size();
@@ -805,11 +806,15 @@ struct DevInfo {
     bool maxl1 = false;  // grid of one CTA per SM without dynamic shared memory: prefer L1
 };
 
+constexpr unsigned PSD_DYN = 200 * 1024;  // shared memory for the PSD blocks that a CTA takes at a time
 template <typename T>
-static size_t dyn_smem(const HostProb& H, int threads, bool tma)
+static size_t dyn_smem(const HostProb& H, int threads, bool tma, int ctas)
 {
     size_t psd = 0;
-    for (int d : H.s) psd = std::max(psd, psd_smem_bytes<T>(d));
+    if (!H.s.empty()) {
+        const PsdPlan p = psd_plan<T>(*std::max_element(H.s.begin(), H.s.end()), (int)H.s.size(), ctas, threads, PSD_DYN);
+        psd = (size_t)p.groups * p.bytes;
+    }
     const size_t stage = tma ? (size_t)(threads / 32) * 2 * tma_stage_bytes<T>() : 0;
     return std::max(psd, stage);
 }
@@ -1052,8 +1057,8 @@ extern "C" int scs_setup(const scs_data* data, const scs_cone* cone, const scs_s
         delete w;
         return SCS_EINVAL;
     }
-    w->D.dyn64 = std::max({dyn_smem<double>(H, w->D.threads, tma), H.cA64.dyn(), H.cAT64.dyn()});
-    w->D.dyn32 = w->has32 ? std::max({dyn_smem<float>(H, w->D.threads, tma), H.cA32.dyn(), H.cAT32.dyn()}) : 0;
+    w->D.dyn64 = std::max({dyn_smem<double>(H, w->D.threads, tma, team == SCS_TEAM_GRID ? w->D.sms : 1), H.cA64.dyn(), H.cAT64.dyn()});
+    w->D.dyn32 = w->has32 ? std::max({dyn_smem<float>(H, w->D.threads, tma, team == SCS_TEAM_GRID ? w->D.sms : 1), H.cA32.dyn(), H.cAT32.dyn()}) : 0;
     // the FP64 phase of SCS_MIXED also runs FP32 products (refinement corrections)
     if (w->has32) w->D.dyn64 = std::max(w->D.dyn64, w->D.dyn32);
     int rc2 = config_kernels<double>(w->err);
