@@ -155,7 +155,7 @@ typedef struct {
                                level is a pause of Algorithm 1, not the FP32 floor; 0: mixed_stall
                                throughout */
     double psd_recheck_tol; /* SCS_MIXED with PSD cones: every FP32 eigendecomposition of a PSD block
-                               (Sec. 2, cone (ii)) is checked in FP64, ||X V - V L||_F / ||X||_F; a
+                               (Sec. 2, cone (ii)) is checked in at least FP64, ||X V - V L||_F / ||X||_F; a
                                block above this bound is decomposed again in FP64 and projected from
                                that.  Default 1e-4, ten times the largest residual of converged FP32
                                Jacobi sweeps on order-64 blocks; 0 redoes every block; must be >= 0 */
