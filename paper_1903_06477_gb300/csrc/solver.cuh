@@ -10,6 +10,8 @@
 // HSDE vectors keep their tau entry in FP64 whatever T is.
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 #include "team.cuh"
 
@@ -185,6 +187,7 @@ struct DevProb {
     const long long* big_off;
     const long long* v_off;  // byte offset of each PSD block's warm-start eigenvectors in DevWork::psd_v
     int psd_order;           // the largest PSD order
+    int psd_small;           // the largest one up to PSD_MAX (0: none)
 };
 
 // Iterative refinement of the FP64 linear solves (SCS_MIXED, FP64 phase): the
@@ -2095,7 +2098,7 @@ __host__ __device__ constexpr size_t psd_matrix_bytes(int dp)  // matrices of on
            (sizeof(T) == 4 ? psd_round(sizeof(double) * (size_t)dp * (dp + 1)) : 0);
 }
 __host__ __device__ constexpr size_t psd_scratch_bytes(int dp) { return sizeof(double) * (64 + 10 * (size_t)dp); }
-// dynamic shared memory of a CTA that projects blocks of order d
+// dynamic shared memory of a CTA that projects a block of order d; not monotone: largest at PSD_MAX
 template <typename T>
 __host__ __device__ constexpr size_t psd_smem_bytes(int d)
 {
@@ -2117,7 +2120,8 @@ __host__ __device__ constexpr size_t psd_v_bytes(int d)
 
 // How a CTA of `threads` threads shares out its PSD blocks, ns of at most order d over `ctas` CTAs, in at
 // most `limit` bytes of shared memory: several blocks at a time, each by a group of its threads, where a
-// CTA has several.  A round of the Jacobi sweeps is a chain of latencies and a block's matrix is small, so
+// CTA has several.  `small` is the largest order up to PSD_MAX (0: none): beside larger orders, whose
+// matrices are elsewhere, it is what sizes a group's memory.  A round of the Jacobi sweeps is a chain of latencies and a block's matrix is small, so
 // a group of 256 threads is hardly slower than 512 (order 64 in FP32, 512 blocks, one group a CTA: 4.0
 // and 3.65 ms; in FP64, where more warps only crowd the pipe, 13.7 and 17.3 ms) and 128 do for small
 // orders (20: 1.01 and 1.10 ms).  A CTA with one block gives it 256 threads, FP32 above order 48 all.
@@ -2126,9 +2130,10 @@ struct PsdPlan {
     unsigned bytes;  // of one group
 };
 template <typename T>
-__host__ __device__ inline PsdPlan psd_plan(int d, int ns, int ctas, int threads, unsigned limit)
+__host__ __device__ inline PsdPlan psd_plan(int d, int small, int ns, int ctas, int threads, unsigned limit)
 {
-    PsdPlan p{threads, 1, (unsigned)psd_smem_bytes<T>(d)};
+    const size_t top = psd_smem_bytes<T>(d), mid = psd_smem_bytes<T>(small);
+    PsdPlan p{threads, 1, (unsigned)(top > mid ? top : mid)};
     if (d > PSD_MAX || ns == 0) return p;
     const int per = (ns + ctas - 1) / ctas;
     int t = d <= 24 ? 128 : 256;
@@ -2139,6 +2144,15 @@ __host__ __device__ inline PsdPlan psd_plan(int d, int ns, int ctas, int threads
     p.groups = room < most ? (room > 1 ? room : 1) : most;
     return p;
 }
+// the orders that size it: the largest, and the largest up to PSD_MAX (0: none)
+inline void psd_orders(const std::vector<int>& orders, int& order, int& small)
+{
+    order = small = 0;
+    for (int d : orders) {
+        order = d > order ? d : order;
+        small = d <= PSD_MAX && d > small ? d : small;
+    }
+}
 __device__ __forceinline__ unsigned dyn_smem_size()
 {
     unsigned n;
@@ -2148,7 +2162,7 @@ __device__ __forceinline__ unsigned dyn_smem_size()
 
 // smem: the CTA's shared region; big: the block's global workspace, or null
 template <typename T>
-__device__ PsdSmem<T> psd_layout(unsigned char* smem, unsigned char* big, int dp)
+__host__ __device__ PsdSmem<T> psd_layout(unsigned char* smem, unsigned char* big, int dp)
 {
     PsdSmem<T> s;
     s.red = (double*)smem;
@@ -2174,7 +2188,7 @@ struct PsdCheck {
     long long* redo;
     double tol;
     // warm starts: block k's eigenvectors of its last converged decomposition are kept at
-    // vbase + voff[k] bytes (dp x (dp+1) elements of the bulk type); vok[k] = 0: none, else the
+    // vbase + voff[k] bytes (dp columns of psd_ldv elements of the bulk type); vok[k] = 0: none, else the
     // number of decompositions since the last cold one
     unsigned char* vbase;
     const long long* voff;
@@ -2274,12 +2288,12 @@ __device__ void project_pass(Team& tm, const DevProb<T>& P, Op& op, unsigned cha
         if (lane == 0) op.store(o + dim - 1, wT, wtT, mode == 0 ? tv : (mode == 1 ? T(0) : (T)tb));
         __syncwarp();
     }
-    // PSD blocks: one group of a CTA's threads per block (psd_groups), Jacobi
+    // PSD blocks: one group of a CTA's threads per block (psd_plan), Jacobi
     // eigen-decomposition in shared memory (orders above PSD_MAX: in the block's
     // workspace in global memory)
     if (P.ns > 0) {
         __syncthreads();  // shared memory is free (earlier users done)
-        const PsdPlan plan = psd_plan<T>(P.psd_order, P.ns, tm.nblocks(), blockDim.x, dyn_smem_size());
+        const PsdPlan plan = psd_plan<T>(P.psd_order, P.psd_small, P.ns, tm.nblocks(), blockDim.x, dyn_smem_size());
         const int gid = threadIdx.x / plan.threads;
         const PsdTeam g{(int)threadIdx.x - gid * plan.threads, plan.threads, 1 + gid};
         const int lane = g.tid & 31, warp = g.tid >> 5, nwb = g.nt >> 5;

@@ -596,7 +596,7 @@ static void lay_out(Arena& A, const HostProb& H, int mem, bool qr, bool direct, 
     P.c = A.take<T>(n);
     P.nb = H.nb;
     P.nc = H.nc;
-    P.psd_order = H.s.empty() ? 0 : *std::max_element(H.s.begin(), H.s.end());
+    psd_orders(H.s, P.psd_order, P.psd_small);
     P.f = H.f;
     P.l = H.l;
     P.nq = (int)H.q.size();
@@ -812,7 +812,9 @@ static size_t dyn_smem(const HostProb& H, int threads, bool tma, int ctas)
 {
     size_t psd = 0;
     if (!H.s.empty()) {
-        const PsdPlan p = psd_plan<T>(*std::max_element(H.s.begin(), H.s.end()), (int)H.s.size(), ctas, threads, PSD_DYN);
+        int order, small;
+        psd_orders(H.s, order, small);
+        const PsdPlan p = psd_plan<T>(order, small, (int)H.s.size(), ctas, threads, PSD_DYN);
         psd = (size_t)p.groups * p.bytes;
     }
     const size_t stage = tma ? (size_t)(threads / 32) * 2 * tma_stage_bytes<T>() : 0;
