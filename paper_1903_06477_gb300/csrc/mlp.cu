@@ -14,6 +14,7 @@
 
 #include <atomic>
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -651,7 +652,10 @@ __global__ void normalize_to_bf16(const float* X, int B, int d, const float* mea
 // A thread has four columns (vec: 16-byte accesses) of LG_ROWS rows.  The
 // squares are summed as exact FP32 products in a two-word (hi, lo) sum, about
 // 48 bits, and in FP64 from there on: adding each square in FP64 took 18 us of
-// the FP64 pipe for 256 x 22004 values, the memory traffic 12 us.
+// the FP64 pipe for 256 x 22004 values, the memory traffic 12 us.  A thread
+// whose sum leaves FP32's range (errors above 1.8e19, infinities, NaN) adds its
+// squares again in FP64.  (Squares below that range, whose low words are lost,
+// are below the FP32 loss's last digit.)
 constexpr int LG_ROWS = 8;
 __global__ void loss_grad(const float* y, const float* tgt, int B, int d, const float* mean, const float* istd,
                           float* dy32, bf16* dy16, int ld16, double* part, int vec)
@@ -704,6 +708,16 @@ __global__ void loss_grad(const float* y, const float* tgt, int B, int d, const 
         }
     }
     double acc = (double)hi + (double)lo;
+    if (!(hi <= FLT_MAX)) {
+        acc = 0.0;
+        for (int r0 = blockIdx.y * LG_ROWS; r0 < B; r0 += (int)gridDim.y * LG_ROWS)
+            for (int r = r0; r < min(B, r0 + LG_ROWS); ++r)
+                for (int k = c; k < min(d, c + 4); ++k) {
+                    const size_t i = (size_t)r * d + k;
+                    const double diff = y[i] - (tgt[i] - mean[k]) * istd[k];
+                    acc += diff * diff;
+                }
+    }
     __shared__ double red[32];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
