@@ -919,7 +919,6 @@ struct scs_mlp {
         int err, pad;
     }* report;              // pinned host copy of (*loss, *err)
     cudaEvent_t reported;   // that copy has arrived
-    bool wt_stale;          // W2t and W3t are older than W2 and W3 (made when needed)
     int step;
     int gemm_impl;  // SCS_MLP_GEMM_MMA or SCS_MLP_GEMM_TCGEN05
     int lastB;      // rows of the last batch that went through forward()
@@ -1300,18 +1299,17 @@ static int refresh_bf16(scs_mlp* n)
     f32_to_bf16_2d<<<grid1d((long long)n->dh * n->din), 256, 0, n->st>>>(n->p + n->oW1, n->dh, n->din, n->W1, n->ldin);
     f32_to_bf16_2d<<<grid1d((long long)n->dh * n->dh), 256, 0, n->st>>>(n->p + n->oW2, n->dh, n->dh, n->W2, n->dh);
     f32_to_bf16_2d<<<grid1d((long long)n->dout * n->dh), 256, 0, n->st>>>(n->p + n->oW3, n->dout, n->dh, n->W3, n->dh);
-    n->wt_stale = true;
     MCU(cudaGetLastError());
     return SCS_OK;
 }
 
-// the transposed copies of W2 and W3: read by the legacy GEMM kernel and by scs_mlp_read only
+// the transposed copies of W2 and W3, made each time they are read, by the legacy GEMM kernel's backward
+// pass or by scs_mlp_read: the host cannot know that they are current, since a captured step updates W2
+// and W3 at every replay
 static void refresh_transposed(scs_mlp* n)
 {
-    if (!n->wt_stale) return;
     transpose(n, n->W2, n->dh, n->dh, n->dh, n->W2t, n->dh);
     transpose(n, n->W3, n->dout, n->dh, n->dh, n->W3t, n->ldout);
-    n->wt_stale = false;
 }
 
 extern "C" int64_t scs_mlp_num_params(const scs_mlp* n) { return n ? n->np : 0; }
@@ -1491,7 +1489,6 @@ extern "C" int scs_mlp_train_step(scs_mlp* n, const float* X, const float* Y, in
     segs.s[4] = {n->oW3, (long long)n->dout * n->dh, n->W3, n->dh, n->dh};
     segs.s[5] = {n->ob3, n->dout, nullptr, 1, 1};
     MCU(launch_next(adam, grid1d((n->np + 3) / 4), 256, 0, n->st, n->p, n->g, n->m, n->v, n->np, lr, b1c, b2c, segs, n->err));
-    n->wt_stale = true;
     if (loss && (rc = report_wait(n, loss))) n->step--;  // Adam saw the error and did nothing
     return rc;
 }
