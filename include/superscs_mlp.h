@@ -44,7 +44,10 @@ int scs_mlp_create(int32_t d_in, int32_t d_hidden, int32_t d_out, int32_t max_ba
 int scs_mlp_fit_normalization(scs_mlp *mlp, const float *X, const float *Y, int64_t rows);
 
 /* One Adam step on a batch (B <= max_batch): forward, loss, backward,
- * update.  *loss (host) receives the batch loss before the update. */
+ * update.  *loss (host) receives the batch loss before the update; with NULL
+ * the step is only queued.  A tensor-core wait that times out (SCS_ECUDA) leaves
+ * the parameters and the step count as they were; of a queued step, and of
+ * those queued behind it, a later call on the network reports it. */
 int scs_mlp_train_step(scs_mlp *mlp, const float *X, const float *Y, int32_t B, float lr, float *loss);
 
 /* Y (B x d_out, FP32, output units) = network(X). */

@@ -777,7 +777,8 @@ __global__ void __launch_bounds__(BS_COLS) bias_sums(const __grid_constant__ Sum
 }
 
 // Adam on all parameters, four at a time (segments start at multiples of 4); refreshes the BF16
-// copies of the weight matrices.  Does nothing once a GEMM of the step reported an error.
+// copies of the weight matrices.  Does nothing once a GEMM of this step or an earlier one reported an
+// error, and then says so in *skipped (host memory); else counts the step in *applied.
 // Bound by memory: 7 words and a BF16 copy a parameter, 0.77 GB for 25.6 M of them, 115 us at the
 // copy rate; one element a thread with a search of its segment took 199 us.
 struct Seg {
@@ -790,10 +791,15 @@ struct Segs {
     Seg s[6];
 };
 __global__ void __launch_bounds__(256) adam(float* p, const float* g, float* m, float* v, long long n, float lr, float b1c,
-                                            float b2c, Segs segs, const int* err)
+                                            float b2c, Segs segs, const int* err, int* applied, int* skipped)
 {
     after_predecessor();
-    if (*err) return;
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (*err) {
+        if (first) *(volatile int*)skipped = 1;
+        return;
+    }
+    if (first) ++*applied;
     auto step = [&](float pi, float gi, float& mi, float& vi) {
         mi = 0.9f * mi + 0.1f * gi;
         vi = 0.999f * vi + 0.001f * gi * gi;
@@ -913,13 +919,15 @@ struct scs_mlp {
     bf16 *Xn, *Xnt, *h1, *h1t, *h2, *h2t, *dy16, *dyt, *dh2_16, *dh2t, *dh1_16, *dh1t;
     float *y, *dy32, *dh2_32, *dh1_32;
     double *part, *loss;
-    int* err;  // set by a tensor-core GEMM whose bounded wait expired; beside *loss, so one copy reads both
+    int* err;  // set by a tensor-core GEMM whose bounded wait expired; beside *loss, so one copy reads all three
+    int* applied;           // Adam steps made
     struct Report {
         double loss;
-        int err, pad;
-    }* report;              // pinned host copy of (*loss, *err)
+        int err, applied;
+    }* report;              // pinned host copy of (*loss, *err, *applied)
     cudaEvent_t reported;   // that copy has arrived
-    int step;
+    int* skipped;           // pinned, beside it: set by an Adam step that found *err set and did nothing
+    int step;               // Adam steps queued; those made, after an error
     int gemm_impl;  // SCS_MLP_GEMM_MMA or SCS_MLP_GEMM_TCGEN05
     int lastB;      // rows of the last batch that went through forward()
     float* ws;      // split-K partial tiles of the tensor-core GEMMs
@@ -1158,20 +1166,26 @@ static int gemm(scs_mlp* n, int M, int N, int K, const bf16* A, int lda, bool am
 {
     return launch_gemm(n->gemm_impl, n->st, n->err, M, N, K, A, lda, amn, B, ldb, bmn, e, n->ws, n->ws_floats);
 }
-// reads (and clears) the tensor-core GEMM's timeout flag; the stream must be synchronised
+// Waits for the stream and reads (and clears) the tensor-core GEMMs' timeout flag.  After an error the
+// steps that Adam skipped no longer count.
 static int check_err_flag(scs_mlp* n)
 {
-    int h = 0;
-    MCU(cudaMemcpyAsync(&h, n->err, sizeof(int), cudaMemcpyDeviceToHost, n->st));
+    scs_mlp::Report r{};
+    MCU(cudaMemcpyAsync(&r, n->loss, sizeof r, cudaMemcpyDeviceToHost, n->st));
     MCU(cudaStreamSynchronize(n->st));
-    if (h) {
+    if (r.err) {
         MCU(cudaMemsetAsync(n->err, 0, sizeof(int), n->st));
-        if (h >= 2) g_tc_fatal = true;
-        sscs::record_error(h >= 2 ? TC_FATAL_MSG : "mlp: a tensor-core GEMM wait timed out; its output tile was not written");
+        n->step = r.applied;
+        *(volatile int*)n->skipped = 0;
+        if (r.err >= 2) g_tc_fatal = true;
+        sscs::record_error(r.err >= 2 ? TC_FATAL_MSG : "mlp: a tensor-core GEMM wait timed out; its output tile was not written");
         return SCS_ECUDA;
     }
     return SCS_OK;
 }
+// An error of an earlier call that did not wait for its own (a step without a loss), once an Adam step has
+// been skipped for it: the host sees it without waiting.
+static int earlier_error(scs_mlp* n) { return *(volatile int*)n->skipped ? check_err_flag(n) : SCS_OK; }
 static void transpose(scs_mlp* n, const bf16* in, int R, int C, int ld_in, bf16* out, int ld_out)
 {
     dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
@@ -1275,10 +1289,13 @@ extern "C" int scs_mlp_create(int32_t din, int32_t dh, int32_t dout, int32_t max
         o += (pl.second + 255) & ~size_t(255);
     }
     n->err = reinterpret_cast<int*>(n->loss + 1);
+    n->applied = n->err + 1;
     auto fail = [&](int rc) { scs_mlp_destroy(n); return rc; };
-    if (cudaMallocHost((void**)&n->report, sizeof(scs_mlp::Report)) != cudaSuccess ||
+    if (cudaMallocHost((void**)&n->report, sizeof(scs_mlp::Report) + sizeof(int)) != cudaSuccess ||
         cudaEventCreateWithFlags(&n->reported, cudaEventDisableTiming) != cudaSuccess)
         return fail(mlp_err("cudaMallocHost", cudaGetLastError()));
+    n->skipped = reinterpret_cast<int*>(n->report + 1);
+    *n->skipped = 0;
     if (cudaMemsetAsync(n->arena, 0, off, n->st) != cudaSuccess) return fail(mlp_err("memset", cudaGetLastError()));
     init_uniform<<<grid1d((long long)dh * din), 256, 0, n->st>>>(n->p, n->oW1, (long long)dh * din, 1.f / sqrtf((float)din), seed);
     init_uniform<<<grid1d((long long)dh * dh), 256, 0, n->st>>>(n->p, n->oW2, (long long)dh * dh, 1.f / sqrtf((float)dh), seed);
@@ -1429,7 +1446,7 @@ static int backward(scs_mlp* n, const float* Y, int B)
     return SCS_OK;
 }
 
-// queues the copy of (*loss, *err) to the host; report_wait reads it once it has arrived
+// queues the copy of (*loss, *err, *applied) to the host; report_wait reads it once it has arrived
 static int report_queue(scs_mlp* n)
 {
     MCU(cudaMemcpyAsync(n->report, n->loss, sizeof(scs_mlp::Report), cudaMemcpyDeviceToHost, n->st));
@@ -1450,7 +1467,8 @@ extern "C" int scs_mlp_forward(scs_mlp* n, const float* X, int32_t B, float* Y)
         sscs::record_error("scs_mlp_forward: bad arguments");
         return SCS_EINVAL;
     }
-    return forward(n, X, B, Y);
+    const int rc = earlier_error(n);
+    return rc ? rc : forward(n, X, B, Y);
 }
 
 extern "C" int scs_mlp_gradients(scs_mlp* n, const float* X, const float* Y, int32_t B, float* grad, float* loss)
@@ -1459,7 +1477,8 @@ extern "C" int scs_mlp_gradients(scs_mlp* n, const float* X, const float* Y, int
         sscs::record_error("scs_mlp_gradients: bad arguments");
         return SCS_EINVAL;
     }
-    int rc = forward(n, X, B);
+    int rc = earlier_error(n);
+    if (!rc) rc = forward(n, X, B);
     if (!rc) rc = backward(n, Y, B);
     if (rc) return rc;
     if (grad) MCU(cudaMemcpyAsync(grad, n->g, sizeof(float) * n->np, cudaMemcpyDefault, n->st));
@@ -1473,7 +1492,8 @@ extern "C" int scs_mlp_train_step(scs_mlp* n, const float* X, const float* Y, in
         sscs::record_error("scs_mlp_train_step: bad arguments");
         return SCS_EINVAL;
     }
-    int rc = forward(n, X, B);
+    int rc = earlier_error(n);
+    if (!rc) rc = forward(n, X, B);
     if (!rc) rc = backward(n, Y, B);
     // the loss is on its way before Adam runs, so that the next step can be queued under it
     if (!rc && loss) rc = report_queue(n);
@@ -1488,9 +1508,9 @@ extern "C" int scs_mlp_train_step(scs_mlp* n, const float* X, const float* Y, in
     segs.s[3] = {n->ob2, n->dh, nullptr, 1, 1};
     segs.s[4] = {n->oW3, (long long)n->dout * n->dh, n->W3, n->dh, n->dh};
     segs.s[5] = {n->ob3, n->dout, nullptr, 1, 1};
-    MCU(launch_next(adam, grid1d((n->np + 3) / 4), 256, 0, n->st, n->p, n->g, n->m, n->v, n->np, lr, b1c, b2c, segs, n->err));
-    if (loss && (rc = report_wait(n, loss))) n->step--;  // Adam saw the error and did nothing
-    return rc;
+    MCU(launch_next(adam, grid1d((n->np + 3) / 4), 256, 0, n->st, n->p, n->g, n->m, n->v, n->np, lr, b1c, b2c, segs, n->err,
+                    n->applied, n->skipped));
+    return loss ? report_wait(n, loss) : SCS_OK;
 }
 
 extern "C" int scs_mlp_set_gemm(scs_mlp* n, int32_t impl)
