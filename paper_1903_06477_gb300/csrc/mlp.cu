@@ -1274,7 +1274,9 @@ extern "C" int scs_mlp_create(int32_t din, int32_t dh, int32_t dout, int32_t max
     take((void**)&n->dh1_32, sizeof(float) * (size_t)maxB * dh);
     take((void**)&n->part, sizeof(double) * (size_t)loss_grid(dout, maxB).x * loss_grid(dout, maxB).y);
     take((void**)&n->loss, sizeof(scs_mlp::Report));
-    // split-K workspace: up to 20 partial sums of a batch-row product (256 x 1024: 19 fill the SMs)
+    // split-K workspace: 20 partial sums of a max_batch-row product, room for the 19 ranges that fill 152 SMs
+    // with the 8 tiles of up to 128 rows by 1024 columns (256 rows take 10); thinner products get fewer ranges
+    // than would fill the SMs
     n->ws_floats = (size_t)20 * maxB * (size_t)std::max(std::max(dh, din), 128);
     take((void**)&n->ws, sizeof(float) * n->ws_floats);
     for (auto& pl : plan) off += (pl.second + 255) & ~size_t(255);
