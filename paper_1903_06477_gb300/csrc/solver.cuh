@@ -531,7 +531,11 @@ __device__ __forceinline__ void cb_segment(int nw, unsigned mt_off, unsigned xs_
                 if (r != 0xFFFF) acc[r] += a;
             }
         } else {
-            // FP64: two chains
+            // FP64: two chains.  The row index is read ahead of them: after the sum, with H (lanes per row) in a
+            // register only since the segments choose it, it cost the product 1 us (1e7 nonzeros, A, A^T and a CG
+            // iteration: 41.1, 44.0 and 93.6 us with one H for the matrix, 43.3, 45.0 and 95.4 with H by segment,
+            // 42.5, 44.5 and 94.0 so)
+            const int r = lane < H ? sr[s * H + lane] : 0xFFFF;
             T a0 = 0, a1 = 0;
             for (; t + 2 <= t1; t += 2) {
                 const int c0 = scol[t * 32 + lane], c1 = scol[t * 32 + 32 + lane];
@@ -542,10 +546,7 @@ __device__ __forceinline__ void cb_segment(int nw, unsigned mt_off, unsigned xs_
             if (t < t1) a0 = fmaT(sval[t * 32 + lane], xs[scol[t * 32 + lane]], a0);
             T a = a0 + a1;
             for (int o = H; o < 32; o <<= 1) a += __shfl_xor_sync(FULL_MASK, a, o);
-            if (lane < H) {
-                const int r = sr[s * H + lane];
-                if (r != 0xFFFF) acc[r] += a;
-            }
+            if (r != 0xFFFF) acc[r] += a;
         }
     }
 }
