@@ -373,7 +373,7 @@ def run_batch(args):
     costs = [shard.instance_cost(p) for p in probs_all]
     mine = shard.partition(costs, world)[rank]
     probs = [probs_all[i] for i in mine]
-    # linear systems by the dense inverse of I + A^T A (n <= 401 here): 10.1k solves/s against
+    # linear systems by the dense factor of I + A^T A (n <= 401 here): 10.1k solves/s against
     # 5.9k with CG, whose inexact solves also cost more outer iterations (median 242 against 178)
     kw = dict(direction=0, mem=10, eps=1e-5, max_iters=20000, cg_rtol=1e-10, cg_adapt=1e-2, mixed_switch=1e-5,
               linsys_direct=1)
@@ -463,7 +463,7 @@ def run_batch(args):
             "vs_baseline": None, "dtype": "f32+f64" if prec == B.MIXED else "f64", "data": "synthetic",
             "config": {"workload": f"{len(probs_all)} portfolio SOCPs, k ~ U{{20..400}}, rank k/10, eps 1e-5, "
                                    f"AA mem 10", "precision": args.precision, "instances": len(probs_all),
-                       "linsys": "direct (dense inverse of I + A^T A)" if kw.get("linsys_direct") else "CG",
+                       "linsys": "direct (inverse of the dense Cholesky factor of I + A^T A)" if kw.get("linsys_direct") else "CG",
                        "nnz_total": int(sum(p["A"].nnz for p in probs_all)),
                        "parallelism": f"instances sharded over {world} GPUs by nnz+n+m" if world > 1 else "single",
                        "l2": "the batch's data (about 0.3 GB with both precisions) exceeds L2"},
@@ -778,7 +778,7 @@ def main():
     ap.add_argument("--spmv-path", type=int, default=None,
                     help="grid-team sparse products: 0 automatic, 1/2 sliced ELL, 3 column-blocked, 4 tiles")
     ap.add_argument("--linsys-direct", type=int, default=None,
-                    help="1: block-team instances solve their linear systems by a dense inverse")
+                    help="1: block-team instances solve their linear systems by a dense factor")
     ap.add_argument("--mixed-refine", type=int, default=None,
                     help="1: the FP64 phase solves by iterative refinement with FP32 corrections")
     ap.add_argument("--instances", type=int, default=4096, help="batch size of the c4 workload")

@@ -142,10 +142,10 @@ typedef struct {
                                corrections by CG with the FP32 copy -- so its FP64 work is a few
                                sparse products per solve; 0: plain FP64 CG */
     int32_t linsys_direct;  /* 1: instances run by one thread block (the block team, every batch
-                               instance) with n <= 4096 form I + A^T A densely at setup, invert it
-                               in each precision (a "direct" solve as Sec. 4.1 names beside CG)
-                               and solve each linear system by one symmetric product; the
-                               inverse takes n^2 words per precision.  0 (default): CG.  Ignored by
+                               instance) with n <= 4096 form I + A^T A densely at setup, factor it
+                               L L^T and invert L in each precision (a "direct" solve as Sec. 4.1
+                               names beside CG) and solve each linear system by two triangular
+                               products; L^{-1} and its transpose take n^2 words per precision.  0 (default): CG.  Ignored by
                                the grid team.  A non-positive pivot makes setup fail with SCS_EINVAL */
     int32_t mixed_stall_after_tau; /* SCS_MIXED, 1 (default): while the FP32 phase's termination test
                                sees tau_ = 0, or max(pr, dr, gap) above 100 mixed_switch, its stall

@@ -498,7 +498,7 @@ static void finish_layouts(HostProb& H, bool sell_A, bool sell_T)
     std::vector<double>().swap(H.Tx);
 }
 
-constexpr int DIRECT_MAX_N = 4096;  // largest n inverted densely for the direct linear solves
+constexpr int DIRECT_MAX_N = 4096;  // largest n factored densely for the direct linear solves
 
 static int check_settings(const scs_settings* S, char* err)
 {
@@ -1093,7 +1093,7 @@ extern "C" int scs_setup(const scs_data* data, const scs_cone* cone, const scs_s
     DevWork<float> W32{};
     const int mem = std::max(settings->mem, 1);
     const bool qr = settings->direction == SCS_DIR_AA_QR;
-    // direct solves: one CTA per instance only (the inverse is formed and used by one CTA)
+    // direct solves: one CTA per instance only (the factor is formed and used by one CTA)
     const bool direct = settings->linsys_direct && team == SCS_TEAM_BLOCK && H.n <= DIRECT_MAX_N;
     lay_out<double>(A, H, mem, qr, direct, w->D.grid, P64, W64, nullptr);
     if (w->has32) lay_out<float>(A, H, mem, qr, direct, w->D.grid, P32, W32, (const int*)1);
@@ -1128,7 +1128,7 @@ extern "C" int scs_setup(const scs_data* data, const scs_cone* cone, const scs_s
     if ((rc = upload<double>(H, w->P64, true, w->stream, w->err))) return fail(rc);
     if (w->has32 && (rc = upload<float>(H, w->P32, false, w->stream, w->err))) return fail(rc);
     if (direct) {
-        // invert I + A^T A in each precision before g is solved with it
+        // factor I + A^T A in each precision before g is solved with it
         DevSettings SF = dev_settings(settings);
         if ((rc = launch<double>(w->D, w->D.dyn64, make_args(w->P64, w->W64, SF, MODE_FACTOR), w->dargs64, w->queue,
                                  w->stream, w->err)))
@@ -1150,7 +1150,7 @@ extern "C" int scs_setup(const scs_data* data, const scs_cone* cone, const scs_s
         int f64 = 0, f32 = 0;
         cudaMemcpy(&f64, w->W64.dinv_fail, sizeof(int), cudaMemcpyDeviceToHost);
         if (w->has32) cudaMemcpy(&f32, w->W32.dinv_fail, sizeof(int), cudaMemcpyDeviceToHost);
-        if (f64 || f32) { set_err(w->err, "inversion of I + A^T A met a non-positive pivot"); return fail(SCS_EINVAL); }
+        if (f64 || f32) { set_err(w->err, "Cholesky factorisation of I + A^T A met a non-positive pivot"); return fail(SCS_EINVAL); }
     }
     for (auto& e : w->ev)
         if (cudaEventCreate(&e) != cudaSuccess) { set_err(w->err, "cudaEventCreate failed"); return fail(SCS_ECUDA); }
@@ -1737,7 +1737,7 @@ static int batch_finish_setup(scs_batch* b, const scs_settings* settings, scs_ba
     b->threads = settings->threads ? settings->threads : 256;
     b->grid = occupancy_grid<double>(b->threads, b->dyn64, b->sms, B);
     if (direct) {
-        // invert I + A^T A of every instance (n <= DIRECT_MAX_N) in each precision before g is solved with it
+        // factor I + A^T A of every instance (n <= DIRECT_MAX_N) in each precision before g is solved with it
         CU(cudaMemsetAsync(b->queue, 0, sizeof(int), b->stream), b->err);
         CU(launch_block<double>(block_kernel<double>(b->threads, b->dyn64, b->sms, B), b->grid, b->threads, b->dyn64, b->stream, b->d64, B, b->queue, S64, MODE_FACTOR), b->err);
         if (b->has32) {
