@@ -1629,8 +1629,8 @@ extern "C" int scs_mlp_read(scs_mlp* n, int32_t what, void* out, int64_t* rows, 
 extern "C" void scs_mlp_destroy(scs_mlp* n)
 {
     if (!n) return;
+    if (n->arena) cudaFree(n->arena);  // waits for the device: a queued step may still write the pinned report
     if (n->reported) cudaEventDestroy(n->reported);
     if (n->report) cudaFreeHost(n->report);
-    if (n->arena) cudaFree(n->arena);
     delete n;
 }
