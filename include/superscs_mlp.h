@@ -111,9 +111,10 @@ void scs_mlp_destroy(scs_mlp *mlp);
 int scs_mlp_read(scs_mlp *mlp, int32_t what, void *out, int64_t *rows, int64_t *cols, int32_t *elem_bytes);
 
 /* GEMM kernels of the network.  SCS_MLP_GEMM_TCGEN05 (the default):
- * fifth-generation tensor cores (tcgen05.mma, accumulator in tensor memory),
- * 128 x 128 tiles fed by TMA from tensor maps (128-byte swizzle, a four-stage
- * ring, producer / MMA / epilogue warps), K split across CTAs with a
+ * fifth-generation tensor cores (tcgen05.mma, accumulators in tensor memory),
+ * tiles of 128 or 256 rows by 32 to 256 columns fed by TMA from tensor maps
+ * (128-byte swizzle, a ring of two to eight stages, producer / MMA / epilogue
+ * warps), operands stored K- or row-contiguous, K split into ranges with a
  * fixed-order reduction when the tiles alone would leave most SMs idle.
  * SCS_MLP_GEMM_MMA: warp-level BF16 MMA (m16n8k16) from shared memory.  Both
  * compute C = A B^T in FP32 from BF16 operands; their results differ only in
