@@ -2083,8 +2083,12 @@ static __device__ void expc_project(double& x1, double& x2, double& x3)
     // The grid.  Only the signs of F matter, and they are found in FP32 (the FP64 pipe runs at
     // 1/64 of the FP32 rate): with (r, s, t) scaled to a largest entry of 1, the FP32 value of F
     // is off by less than 8e-6 of the sum of its terms' magnitudes, so where it is larger its
-    // sign is F's; nearer a root F is evaluated in FP64.  The sign changes are noted first and
-    // refined afterwards, so that the lanes of a warp (one cone each) refine theirs together.
+    // sign is F's; nearer a root F is evaluated in FP64.  (A term is an input rounded to FP32, a
+    // polynomial in rho that is exact, since rho is a multiple of 1/4 up to 60, and e or e^2, e
+    // within 2 ulp: at most 8 roundings a term and 4 in the sums, 7e-7 of the magnitudes.  Where
+    // e^2 or an input underflows, its term is below 1e-38 beside one of 3e-23 at least.)  The sign
+    // changes are noted first and refined afterwards, so that the lanes of a warp (one cone each)
+    // refine theirs together.
     const double big = fmax(fabs(r), fmax(fabs(s), fabs(t)));
     const bool scan32 = isfinite(big) && big > 1e-290;
     const double sc = scan32 ? 1.0 / big : 0.0;
