@@ -1557,13 +1557,15 @@ __device__ __forceinline__ double block_sum(double x, double* red, const PsdTeam
 // is found in FP32 -- any t with c = 1/sqrt(1 + t^2), s = t c is a rotation,
 // and c, the scales and the diagonal are FP64 for the t that was taken; an
 // angle 1e-7 off leaves 1e-7 of the element for the next sweep.  Once the
-// off-diagonal part is below 1e-4 of the whole, a Newton step in FP64 makes
+// off-diagonal part is below 3e-6 of the whole, a Newton step in FP64 makes
 // the angle exact to 1e-14: what the last sweep leaves is the projection's
 // error, and with FP32 angles it stopped just under the test (mean error over
-// |X| of 400 random blocks, by a simulation on the CPU, FP64 angles / FP32
-// angles / so: order 2 1.5e-16, 2.8e-15, 1.1e-16; order 5 2.7e-15, 5.0e-15,
-// 2.1e-15; order 17 4.0e-15, 6.5e-15, 2.8e-15; order 32 6.4e-15, 3.7e-15,
-// 3.4e-15), often after one sweep more.
+// |X| of random blocks, by a simulation on the CPU, FP64 angles / FP32 angles /
+// so: order 2 1.1e-16, 2.7e-15, 1.5e-16; order 5 2.8e-15, 5.5e-15, 1.1e-15;
+// order 17 4.2e-15, 5.2e-15, 3.2e-15; order 32 6.6e-15, 3.8e-15, 3.6e-15),
+// often after one sweep more.  The line lies where a sweep's quadratic remainder
+// begins to fall below 1e-7 of what it started from; at 1e-4 two sweeps of a warm
+// start took the step instead of one (a tenth of a rotation's chain each).
 //
 // V (columns contiguous, stride ldv) receives the eigenvectors; its update is
 // left to the warps that compute no rotations, a round's longest chain.
@@ -1814,7 +1816,7 @@ __device__ __noinline__ bool jacobi_sweeps(const Jacobi<T> J, double* red, doubl
         const double off = block_sum(square_sum(cur), red, g);
         conv = off <= tol2 * total || off == 0.0;
         if (conv || sweep == max_sweeps) break;
-        if constexpr (kFast) fine = off <= 1e-8 * total;
+        if constexpr (kFast) fine = off <= 1e-11 * total;
         for (int k = tid; k < half; k += nt) {
             if constexpr (kFast) {
                 J.sc[cur * dp + 2 * k] = J.sc[cur * dp + 2 * k + 1] = T(1);
