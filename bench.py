@@ -36,8 +36,8 @@ FALLBACK_HBM_GBS = 6800.0
 # it was taken on (the digest of KERNEL_SOURCES) and for the same deterministic
 # solve (same outer and CG iteration counts); otherwise the roofline reports null.
 MEASURED_TRAFFIC = {
-    ("c2", "mixed"): {"bytes": 516166701568, "iters_fp32": 144, "cg_iters": 4251,
-                      "digest": "ab569cbe45e88e3232ad094bdafcbc6e452466d474c3b723457eb56e708fd80c"},
+    ("c2", "mixed"): {"bytes": 519799131392, "iters_fp32": 144, "cg_iters": 4251,
+                      "digest": "f6700325f3d37e72079e675070b531a43dc5ceaf3211f03683479f2ac68aaa62"},
 }
 
 # the sources that decide what the solver kernels do and which bytes they move:
@@ -930,12 +930,12 @@ def main():
                     "note": "the instance lives in one SM's shared memory / L1 and L2; no HBM roofline applies"}
     elif prob.get("s"):
         # PSD blocks: the phase is spent in the Jacobi eigensolves, bound by shared-memory latency and
-        # CTA barriers (ncu: FP32 FMA pipe 13.5%, DRAM 58 GB/s); the HBM figures are kept for reference
+        # barriers (ncu: FP32 FMA pipe 17.2%, DRAM 224 GB/s); the HBM figures are kept for reference
         roofline = {"bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None,
                     "traffic": None, "kernel": kname, "kernel_ms": ks * 1e3,
                     "hbm_achieved_gbs": achieved, "hbm_frac": achieved / peak,
-                    "note": "PSD projections dominate: parallel Jacobi sweeps in shared memory, one CTA barrier "
-                            "per half-round; neither DRAM- nor ALU-bound"}
+                    "note": "PSD projections dominate: parallel Jacobi sweeps in shared memory, one barrier "
+                            "per round; neither DRAM- nor ALU-bound"}
     else:
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": traffic, "peak_source": peak_kind, "kernel": kname,
