@@ -1547,7 +1547,8 @@ __device__ __forceinline__ double block_sum(double x, double* red, const PsdTeam
 // matrix with a barrier each: 4400 cycles a round for order 64 in FP32, 12000 in
 // FP64; one pass over the indexed lower triangle: 2400 and 10800; the cells: 1160
 // and 6540.  512 blocks of order 64 in FP32, one projection: 10.0, 6.5 and 4.6 ms;
-// one block of order 120 in FP64, four iterations: 129, 76 and 42 ms.)
+// one block of order 120 in FP64, four iterations: 129, 76 and 42 ms, 45 with the
+// sweeps out of line.)
 //
 // FP64: the FP64 pipe (2 multiply-adds a cycle and SM) is the bound, so the
 // rotations are applied in scaled form (fast Givens): X = D X^ D and V = V^ D
@@ -1637,7 +1638,8 @@ __device__ __forceinline__ float jacobi_tan(float diff, float apq)
 // thread); dg[slot_of(i)] of buffer `cur` then is eigenvalue i.
 //
 // A function of its own: inlined at its five places it made the solver's kernels so large that their
-// other loops ran slower (sparse program of 1e7 nonzeros in FP64, ten iterations: 28.3 ms, 27.4 ms so).
+// other loops ran slower (sparse program of 1e7 nonzeros in FP64, ten iterations: 28.3 ms, 27.4 ms so; 27.1 since
+// a slice's row index is read ahead).
 template <typename T>
 __device__ __noinline__ bool jacobi_sweeps(const Jacobi<T> J, double* red, double tol2, int max_sweeps, int& cur,
                                            const PsdTeam g)
